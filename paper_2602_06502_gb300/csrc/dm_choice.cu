@@ -19,6 +19,8 @@
 // with the hits on every live instance probed beforehand by k_probe_all.
 //
 // At the end of the file: routing with d candidates (App. A.8).
+#include <algorithm>
+
 #include "dm_internal.cuh"
 
 namespace dm {
@@ -88,13 +90,121 @@ __device__ void finish_metrics(const DevState &d, uint32_t n, MetricSums ms, uns
 }
 
 
-constexpr uint32_t kChoiceChunk = 1024;
-
-// Single CTA (1024 threads).  Dynamic shared memory: per instance W (u64),
-// a packed counter PT = (log records this batch << 32) | queue tail, so one
-// 64-bit add per request advances both, and a lane mask used to find
-// conflicts inside a window; then the per-chunk request staging.
+// ---------------------------------------------------------------------------
+// Choices in arrival order, pipelined over chunks of requests.
 //
+// What bounds a choice kernel is the chain of decisions that share an
+// instance: on batches of hot templates about a third of the requests follow
+// one another through the same pair.  So one warp does nothing but decide,
+// and everything else is kept out of its way:
+//   stage   a warp per window of 32 requests loads the requests and finds
+//           each one's level, 1 + the largest level of the earlier requests
+//           of its window that share an instance with it.  The levels depend
+//           on the candidates alone, so they are known before any decision;
+//   decide  warp 0, window by window, level by level: requests of one level
+//           share no instance, so reading W and writing W[choice] for all of
+//           them at once equals arrival order exactly.  A level is two loads,
+//           a compare and a store in shared memory: no vote, no branch on
+//           what is done;
+//   emit    a warp per window places the requests among their instances'
+//           records and queue entries and writes every output.
+// Chunk t is staged while chunk t - 1 is decided and chunk t - 2 emitted,
+// over three staging buffers.  Measured (GB300, a routed and committed pass
+// of 4,096 agent prompts): 311 us when windows were decided in rounds found
+// by votes, by the warp that also kept the record counters, with staging,
+// deciding and emitting one after the other; 255 us so.  The d-candidate
+// choice, one thread from global memory before: 5,360 and 577 us (d = 4).
+constexpr uint8_t kNoLevel = 255;
+
+template <uint32_t kChunk>
+struct Pipe {
+    static constexpr uint32_t kWindows = kChunk / 32;
+    static constexpr uint32_t kThreads = 32 + 2 * kChunk;   // warp 0, the emitting warps, the staging warps
+};
+
+// stage(buffer, k, m, base), decide(buffer, m), emit(buffer, k, m, base): k
+// this thread's request of the chunk (whole windows call; k >= m past the
+// batch's end), m its requests, base its first request.
+template <uint32_t kChunk, class StageF, class DecideF, class EmitF>
+__device__ __forceinline__ void choice_pipeline(uint32_t n, StageF stage, DecideF decide, EmitF emit) {
+    const uint32_t nc = (n + kChunk - 1) / kChunk, tid = threadIdx.x;
+    for (uint32_t t = 0; t < nc + 2; ++t) {
+        if (tid < 32) {
+            if (t >= 1 && t <= nc) decide((t - 1) % 3, min(kChunk, n - (t - 1) * kChunk));
+        } else if (tid < 32 + kChunk) {
+            if (t >= 2) emit((t - 2) % 3, tid - 32, min(kChunk, n - (t - 2) * kChunk), (t - 2) * kChunk);
+        } else {
+            if (t < nc) stage(t % 3, tid - 32 - kChunk, min(kChunk, n - t * kChunk), t * kChunk);
+        }
+        __syncthreads();
+    }
+}
+
+// Level of this lane's request in its window (0 first; valid: there is one),
+// from the candidates of all lanes packed in c (kWords words, two 16-bit ids
+// each; unused halves 0xFFFF).  Whole warp; returns also the window's number
+// of levels.
+template <int kWords>
+__device__ __forceinline__ uint32_t window_levels(const uint32_t (&c)[kWords], bool valid, int lane,
+                                                  uint32_t &nlev) {
+    uint32_t lev = 0;
+    const uint32_t vm = __ballot_sync(0xffffffffu, valid);
+    for (int j = 0; j < 31; ++j) {
+        uint32_t o[kWords];
+        bool hit = false;
+#pragma unroll
+        for (int x = 0; x < kWords; ++x) o[x] = __shfl_sync(0xffffffffu, c[x], j);
+#pragma unroll
+        for (int x = 0; x < kWords; ++x) {
+#pragma unroll
+            for (int y = 0; y < kWords; ++y) {   // a set half-word of vcmpeq: an id both name
+                const uint32_t sw = __byte_perm(o[y], 0, 0x1032);
+                hit |= ((__vcmpeq2(c[x], o[y]) | __vcmpeq2(c[x], sw)) & ~__vcmpeq2(c[x], 0xFFFFFFFFu)) != 0;
+            }
+        }
+        const uint32_t lj = __shfl_sync(0xffffffffu, lev, j);
+        if (hit && lane > j && ((vm >> j) & 1u)) lev = max(lev, lj + 1);
+    }
+    nlev = __reduce_max_sync(0xffffffffu, valid ? lev + 1 : 0);
+    return lev;
+}
+
+// Place of each request among its instance's records and queue entries:
+// PT[ch] counts both (records of this batch << 32 | queue tail), step = (the
+// request's blocks << 32) + 1.  Returns PT[ch] as the request finds it and
+// moves PT on.  Called by the emitting warps of a chunk, one window each, in
+// window order over a barrier of their own (valid: the lane has a request).
+template <uint32_t kChunk>
+__device__ __forceinline__ uint64_t record_place(uint64_t *PT, uint32_t ch, uint64_t step, bool valid,
+                                                 uint32_t window, uint32_t windows, int lane) {
+    const uint32_t peers = __match_any_sync(0xffffffffu, valid ? ch : 0x80000000u | lane);
+    const uint32_t lower = peers & ((1u << lane) - 1u);
+    // inclusive sum over the peers up to this lane, by pointer jumping
+    int prev = lower ? 31 - __clz(lower) : -1;
+    uint64_t sum = step;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const uint64_t u = shfl_u64(sum, prev & 31);
+        const int pp = __shfl_sync(0xffffffffu, prev, prev & 31);
+        if (prev >= 0) {
+            sum += u;
+            prev = pp;
+        }
+    }
+    const bool last = (peers >> lane) == 1u;
+    uint64_t place = 0;
+    for (uint32_t w = 0; w < windows; ++w) {
+        if (w == window) {
+            const uint64_t p = valid ? PT[ch] : 0;
+            place = p + sum - step;
+            __syncwarp();
+            if (valid && last) PT[ch] = p + sum;
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(kChunk) : "memory");
+    }
+    return place;
+}
+
 // Each request is staged as (a, b): a = the candidate with more cached
 // blocks (c1 on equal hits), u = uncached work on each, and
 // thr = SLO - u_a (-1 when u_a alone exceeds the SLO or the hits are equal),
@@ -103,25 +213,27 @@ constexpr uint32_t kChoiceChunk = 1024;
 // W_a > thr.  The pair variants use the general form: choose b iff
 // W_a > thr and (k_b < k_a or (k_b == k_a and tieb)), with k = W (+ u when
 // the rule compares TTFTs) and tieb set where a tie goes to b (= c1).
+constexpr uint32_t kChoiceChunk = 256;
 struct ChoiceStage {
     uint64_t ua[kChoiceChunk], ub[kChoiceChunk];
     int64_t thr[kChoiceChunk];
-    uint64_t Wa[kChoiceChunk], Wb[kChoiceChunk], pt[kChoiceChunk];
+    uint64_t Wa[kChoiceChunk], Wb[kChoiceChunk];
     uint32_t ab[kChoiceChunk];     // a | b << 14 | (a is c2) << 28 | (hits differ) << 29 | tieb << 30 | addu << 31
-    uint32_t nb[kChoiceChunk];
-    uint8_t pickb[kChoiceChunk];
+    uint32_t nlev[kChoiceChunk / 32];
+    uint8_t lev[kChoiceChunk], pickb[kChoiceChunk];
 };
 
-// W and PT (8 bytes each), the lane masks padded to a multiple of 4 entries
-// so that the staging block starts on a 16-byte boundary for any M.
-__host__ __device__ inline size_t choice_lanes(uint32_t M) { return (size_t(M) + 3) / 4 * 4; }
-size_t choice_smem(uint32_t M) { return size_t(M) * 16 + choice_lanes(M) * 4 + sizeof(ChoiceStage); }
+// W and PT (8 bytes each) per instance, then the staging buffers.
+size_t choice_smem(uint32_t M) { return size_t(M) * 16 + 3 * sizeof(ChoiceStage); }
 
 // kPairRules: the general form (the pair variants and global cache
 // affinity); false compiles DualMap's rule alone.
+//
+// Bound: about 1,250 dependent levels on an agent batch (4,096 requests, 64
+// instances, 200 templates).
 template <bool kPairRules>
-__global__ void __launch_bounds__(1024) k_choice(DevState d, dm_route_out o, uint32_t n, uint64_t seq0,
-                                                 uint64_t t_batch) {
+__global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads) k_choice(DevState d, dm_route_out o, uint32_t n,
+                                                                         uint64_t seq0, uint64_t t_batch) {
     pdl_enter();
     extern __shared__ __align__(16) unsigned char smem[];
     if (has_err(d.err)) return;
@@ -131,22 +243,24 @@ __global__ void __launch_bounds__(1024) k_choice(DevState d, dm_route_out o, uin
     }
     uint64_t *W = reinterpret_cast<uint64_t *>(smem);
     uint64_t *PT = W + d.M;
-    uint32_t *lanes = reinterpret_cast<uint32_t *>(PT + d.M);
-    ChoiceStage &S = *reinterpret_cast<ChoiceStage *>(lanes + choice_lanes(d.M));
-    uint32_t live_bits = 0;   // bit k: instance threadIdx.x + k * blockDim.x is live (M <= 8 * 1024)
+    ChoiceStage *const SB = reinterpret_cast<ChoiceStage *>(PT + d.M);
+    const int lane = threadIdx.x & 31;
+    uint32_t live_bits = 0;   // bit k: instance threadIdx.x + k * blockDim.x is live (M <= 16 * 544)
     for (uint32_t i = threadIdx.x, k = 0; i < d.M; i += blockDim.x, ++k) {
         W[i] = d.W[i];
         PT[i] = d.q_tail[i];
-        lanes[i] = 0;
         live_bits |= uint32_t(d.inst_state[i] == 1) << k;
     }
     const uint64_t cost = d.cost, slo = d.slo;
     const uint32_t rule = kPairRules ? d.rule : uint32_t(DM_RULE_DUALMAP);
     MetricSums ms{0, 0, 0, 0};
-    for (uint32_t base = 0; base < n; base += kChoiceChunk) {
-        const uint32_t m = min(kChoiceChunk, n - base);
-        __syncthreads();
-        for (uint32_t k = threadIdx.x; k < m; k += blockDim.x) {
+
+    auto stage = [&](uint32_t buf, uint32_t k, uint32_t m, uint32_t base) {
+        if ((k & ~31u) >= m) return;   // no request in this window
+        ChoiceStage &S = SB[buf];
+        const bool valid = k < m;
+        uint32_t ids[1] = {0xFFFFFFFFu};
+        if (valid) {
             const uint32_t r = base + k;
             const uint32_t L = d.r_L[r], nblk = d.r_nblk[r];
             const uint32_t h1 = hit_tokens(d.r_m1[r], nblk, d.B), h2 = hit_tokens(d.r_m2[r], nblk, d.B);
@@ -175,115 +289,106 @@ __global__ void __launch_bounds__(1024) k_choice(DevState d, dm_route_out o, uin
             S.thr[k] = thr;
             S.ab[k] = (a2 ? c2 : c1) | ((a2 ? c1 : c2) << 14) | (uint32_t(a2) << 28) | (uint32_t(differ) << 29) |
                       (uint32_t(tieb) << 30) | (uint32_t(addu) << 31);
-            S.nb[k] = nblk;
+            ids[0] = c1 | c2 << 16;
         }
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            // Warp 0 takes 32 requests at a time.  A lane may decide once
-            // every earlier lane sharing one of its candidates has decided;
-            // lanes decided in the same round share no instance, so reading
-            // W and writing W[choice] then equals arrival order exactly.
-            const int lane = threadIdx.x;
-            for (uint32_t w0 = 0; w0 < m; w0 += 32) {
-                const uint32_t k = w0 + lane;
-                const bool valid = k < m;
-                const uint32_t ab = valid ? S.ab[k] : 0;
-                const uint32_t a = ab & 0x3FFF, b = (ab >> 14) & 0x3FFF;
-                if (valid) {
-                    atomicOr(&lanes[a], 1u << lane);
-                    atomicOr(&lanes[b], 1u << lane);
-                }
-                __syncwarp();
-                const uint32_t conf = valid ? (lanes[a] | lanes[b]) & ((1u << lane) - 1) : 0;
-                __syncwarp();
-                if (valid) { lanes[a] = 0; lanes[b] = 0; }
-                const uint64_t ua = valid ? S.ua[k] : 0, ub = valid ? S.ub[k] : 0;
-                const int64_t thr = valid ? S.thr[k] : 0;
-                const bool tieb = (ab >> 30) & 1u;
-                const uint64_t xa = (ab >> 31) ? ua : 0, xb = (ab >> 31) ? ub : 0;
-                const uint64_t inc = valid ? (uint64_t(S.nb[k]) << 32) + 1 : 0;   // PT step of this request
-                uint64_t oWa = 0, oWb = 0, oP = 0;   // the lane's decision, stored once the window is done
-                bool opb = false;
-                uint32_t done = __ballot_sync(0xffffffffu, !valid);
-                while (done != 0xffffffffu) {
-                    const bool ready = !((done >> lane) & 1u) && (conf & ~done) == 0;
-                    if (ready) {
-                        const uint64_t Wa = W[a], Wb = W[b], Pa = PT[a], Pb = PT[b];
-                        bool pb;
-                        if constexpr (kPairRules) {
-                            const uint64_t ka = Wa + xa, kb = Wb + xb;
-                            pb = (int64_t)Wa > thr && (kb < ka || (kb == ka && tieb));
-                        } else {
-                            pb = Wb < Wa && (int64_t)Wa > thr;
-                        }
-                        const uint32_t ch = pb ? b : a;
-                        const uint64_t Pold = pb ? Pb : Pa;
-                        W[ch] = pb ? Wb + ub : Wa + ua;
-                        PT[ch] = Pold + inc;
-                        oWa = Wa;
-                        oWb = Wb;
-                        oP = Pold;
-                        opb = pb;
-                    }
-                    __syncwarp();
-                    done |= __ballot_sync(0xffffffffu, ready);
-                }
-                if (valid) {
-                    S.Wa[k] = oWa;
-                    S.Wb[k] = oWb;
-                    S.pt[k] = oP;
-                    S.pickb[k] = opb;
-                }
-            }
-        }
-        __syncthreads();
-        for (uint32_t k = threadIdx.x; k < m; k += blockDim.x) {
-            const uint32_t r = base + k;
-            const uint32_t ab = S.ab[k];
+        uint32_t nlev;
+        const uint32_t lev = window_levels<1>(ids, valid, lane, nlev);
+        S.lev[k] = valid ? (uint8_t)lev : kNoLevel;
+        if (lane == 0) S.nlev[k / 32] = nlev;
+    };
+
+    auto decide = [&](uint32_t buf, uint32_t m) {
+        ChoiceStage &S = SB[buf];
+        volatile uint64_t *const Wv = W;
+        for (uint32_t w0 = 0; w0 < m; w0 += 32) {
+            const uint32_t k = w0 + lane;
+            const uint32_t mine = S.lev[k], nlev = S.nlev[w0 / 32];
+            const uint32_t ab = mine != kNoLevel ? S.ab[k] : 0;
             const uint32_t a = ab & 0x3FFF, b = (ab >> 14) & 0x3FFF;
-            const bool a_is_c2 = (ab >> 28) & 1, differ = (ab >> 29) & 1;
-            const bool pb = S.pickb[k];
-            const uint32_t ch = pb ? b : a;
-            const uint64_t ta = S.Wa[k] + S.ua[k], tb = S.Wb[k] + S.ub[k];
-            o.ttft1[r] = a_is_c2 ? tb : ta;
-            o.ttft2[r] = a_is_c2 ? ta : tb;
-            const bool sw = differ && (rule == DM_RULE_DUALMAP ? (int64_t)S.Wa[k] > S.thr[k] : pb);
-            o.chosen[r] = ch;
-            o.switched[r] = sw;
-            d.r_final[r] = ch;
-            const uint32_t L = d.r_L[r], nbr = d.r_nblk[r];
-            const uint32_t h1 = hit_tokens(d.r_m1[r], nbr, d.B), h2 = hit_tokens(d.r_m2[r], nbr, d.B);
-            ms.tokens += L;
-            ms.hits += (ch == (a_is_c2 ? b : a)) ? h1 : h2;
-            ms.sw += sw;
-            ms.est += (pb ? tb : ta) <= slo;
-            if (ta > slo && tb > slo) d.info->both_over = 1;
-            d.r_touchoff[r] = S.pt[k] >> 32;          // offset among this batch's records of ch
-            const uint32_t slot = (uint32_t)S.pt[k];
-            if (slot - d.q_head[ch] >= d.Q) {
-                set_err(d.err, DM_ERR_CAPACITY);
-                continue;
+            const uint64_t ua = S.ua[k], ub = S.ub[k];   // past the batch's end: unused
+            const int64_t thr = S.thr[k];
+            const bool tieb = (ab >> 30) & 1u;
+            const uint64_t xa = (ab >> 31) ? ua : 0, xb = (ab >> 31) ? ub : 0;
+            uint64_t oWa = 0, oWb = 0;
+            bool opb = false;
+            for (uint32_t l = 0; l < nlev; ++l) {
+                const uint64_t Wa = Wv[a], Wb = Wv[b];
+                bool pb;
+                if constexpr (kPairRules) {
+                    const uint64_t ka = Wa + xa, kb = Wb + xb;
+                    pb = (int64_t)Wa > thr && (kb < ka || (kb == ka && tieb));
+                } else {
+                    pb = Wb < Wa && (int64_t)Wa > thr;
+                }
+                const uint64_t na = Wa + ua, nb = Wb + ub;
+                if (mine == l) {
+                    Wv[pb ? b : a] = pb ? nb : na;
+                    oWa = Wa;
+                    oWb = Wb;
+                    opb = pb;
+                }
+                __syncwarp();
             }
-            QEntry e;
-            e.seq = seq0 + r;
-            e.work = e.remaining = pb ? S.ub[k] : S.ua[k];
-            e.L = L;
-            e.c1 = a_is_c2 ? b : a;
-            e.c2 = a_is_c2 ? a : b;
-            e.h1 = h1;
-            e.h2 = h2;
-            e.moved = 0;
-            e.arrival = t_batch;
-            // its keys' ring position: the instance's ring tail at the batch's
-            // start plus this batch's earlier blocks queued there (the same
-            // order as its touch records)
-            e.koff = d.KQ ? d.kr_tail[ch] + (S.pt[k] >> 32) : 0;
-            if (d.KQ) d.r_koff[r] = e.koff;
-            DM_CHECK(ch < d.M, d.err);
-            d.q[uint64_t(ch) * d.Q + (slot & (d.Q - 1))] = e;
+            S.Wa[k] = oWa;
+            S.Wb[k] = oWb;
+            S.pickb[k] = opb;
         }
-    }
+    };
+
+    auto emit = [&](uint32_t buf, uint32_t k, uint32_t m, uint32_t base) {
+        const ChoiceStage &S = SB[buf];
+        const bool valid = k < m;
+        const uint32_t r = base + k;
+        const uint32_t ab = valid ? S.ab[k] : 0;
+        const uint32_t a = ab & 0x3FFF, b = (ab >> 14) & 0x3FFF;
+        const bool a_is_c2 = (ab >> 28) & 1, differ = (ab >> 29) & 1;
+        const bool pb = valid && S.pickb[k];
+        const uint32_t ch = pb ? b : a;
+        const uint32_t nbr = valid ? d.r_nblk[r] : 0;
+        const uint64_t pt = record_place<kChoiceChunk>(PT, ch, (uint64_t(nbr) << 32) + 1, valid, k / 32,
+                                                       (m + 31) / 32, lane);
+        if (!valid) return;
+        const uint64_t ta = S.Wa[k] + S.ua[k], tb = S.Wb[k] + S.ub[k];
+        o.ttft1[r] = a_is_c2 ? tb : ta;
+        o.ttft2[r] = a_is_c2 ? ta : tb;
+        const bool sw = differ && (rule == DM_RULE_DUALMAP ? (int64_t)S.Wa[k] > S.thr[k] : pb);
+        o.chosen[r] = ch;
+        o.switched[r] = sw;
+        d.r_final[r] = ch;
+        const uint32_t L = d.r_L[r];
+        const uint32_t h1 = hit_tokens(d.r_m1[r], nbr, d.B), h2 = hit_tokens(d.r_m2[r], nbr, d.B);
+        ms.tokens += L;
+        ms.hits += (ch == (a_is_c2 ? b : a)) ? h1 : h2;
+        ms.sw += sw;
+        ms.est += (pb ? tb : ta) <= slo;
+        if (ta > slo && tb > slo) d.info->both_over = 1;
+        d.r_touchoff[r] = pt >> 32;          // offset among this batch's records of ch
+        const uint32_t slot = (uint32_t)pt;
+        if (slot - d.q_head[ch] >= d.Q) {
+            set_err(d.err, DM_ERR_CAPACITY);
+            return;
+        }
+        QEntry e;
+        e.seq = seq0 + r;
+        e.work = e.remaining = pb ? S.ub[k] : S.ua[k];
+        e.L = L;
+        e.c1 = a_is_c2 ? b : a;
+        e.c2 = a_is_c2 ? a : b;
+        e.h1 = h1;
+        e.h2 = h2;
+        e.moved = 0;
+        e.arrival = t_batch;
+        // its keys' ring position: the instance's ring tail at the batch's
+        // start plus this batch's earlier blocks queued there (the same
+        // order as its touch records)
+        e.koff = d.KQ ? d.kr_tail[ch] + (pt >> 32) : 0;
+        if (d.KQ) d.r_koff[r] = e.koff;
+        DM_CHECK(ch < d.M, d.err);
+        d.q[uint64_t(ch) * d.Q + (slot & (d.Q - 1))] = e;
+    };
+
     __syncthreads();
+    choice_pipeline<kChoiceChunk>(n, stage, decide, emit);
     unsigned __int128 S1 = 0, S2 = 0;
     uint32_t cnt = 0;
     for (uint32_t i = threadIdx.x, k = 0; i < d.M; i += blockDim.x, ++k) {
@@ -561,11 +666,12 @@ cudaError_t launch_choice(const DevState &d, const dm_route_out &o, uint32_t n, 
         configured = smem;
     }
     // CTA 0 decides; CTAs 1.. sum the batch's segment carries meanwhile (a warp per request)
-    const unsigned grid = 1 + (n + 31) / 32 < 1 + 152 ? 1 + (n + 31) / 32 : 1 + 152;
+    constexpr unsigned threads = Pipe<kChoiceChunk>::kThreads, per = threads / 32;
+    const unsigned grid = 1 + std::min((n + per - 1) / per, 2u * 152u);
     if (d.rule == DM_RULE_DUALMAP)
-        DM_TRY(launch_pdl(k_choice<false>, grid, 1024, smem, st, d, o, n, seq0, t_batch));
+        DM_TRY(launch_pdl(k_choice<false>, grid, threads, smem, st, d, o, n, seq0, t_batch));
     else
-        DM_TRY(launch_pdl(k_choice<true>, grid, 1024, smem, st, d, o, n, seq0, t_batch));
+        DM_TRY(launch_pdl(k_choice<true>, grid, threads, smem, st, d, o, n, seq0, t_batch));
     return cudaGetLastError();
 }
 
@@ -581,10 +687,9 @@ cudaError_t launch_choice(const DevState &d, const dm_route_out &o, uint32_t n, 
 //               distinct fix, and the leading run of resident blocks on
 //               each candidate;
 //   k_choice_d  one CTA: DualMap's SLO-aware rule over d candidates in
-//               arrival order (one thread; this path is for experiments,
-//               not the benchmark), queue appends, the commit's per-request
-//               offsets and the batch's metrics, exactly as k_choice leaves
-//               them for d = 2.
+//               arrival order (the choice pipeline), queue appends, the
+//               commit's per-request offsets and the batch's metrics,
+//               exactly as k_choice leaves them for d = 2.
 
 
 // Index (level 0) of the successor of p on ring f.  Whole warp.
@@ -673,88 +778,184 @@ __global__ void k_route_d(DevState d, const uint32_t *tokens, uint32_t n) {
     if (lane == 0) d.r_K[r] = K;
 }
 
-// DualMap's rule over d candidates, in arrival order (one thread), then the
-// batch's loads, queue tails, commit offsets and metrics as k_choice leaves
-// them.  Dynamic shared memory: W and the packed (records << 32 | queue
-// tail) counter of every instance.
-__global__ void __launch_bounds__(1024) k_choice_d(DevState d, dm_route_out_d o, uint32_t n, uint64_t seq0,
-                                                   uint64_t t_batch) {
+// Staging of one chunk: candidates, uncached work on each, the load of each
+// as the request found it, which candidates have the most hit tokens.
+template <uint32_t ND, uint32_t kChunk>
+struct ChoiceStageD {
+    uint64_t u[ND][kChunk], Wf[ND][kChunk];
+    uint16_t c[ND][kChunk];
+    uint8_t most[kChunk];             // bit f: candidate f has the most hit tokens
+    uint8_t lev[kChunk], pick[kChunk], over[kChunk];
+    uint32_t nlev[kChunk / 32];
+};
+constexpr uint32_t choice_d_chunk(uint32_t nd) { return nd <= 4 ? 256 : 128; }   // three buffers beside 8,192 instances
+
+// DualMap's rule over ND candidates, in arrival order (the pipeline above),
+// then the batch's loads, queue tails, commit offsets and metrics as
+// k_choice leaves them.  Dynamic shared memory: W and the packed (records
+// << 32 | queue tail) counter of every instance, then the staging buffers.
+template <uint32_t ND>
+__global__ void __launch_bounds__(Pipe<choice_d_chunk(ND)>::kThreads) k_choice_d(DevState d, dm_route_out_d o,
+                                                                                 uint32_t n, uint64_t seq0,
+                                                                                 uint64_t t_batch) {
     pdl_enter();
     extern __shared__ __align__(16) unsigned char smem[];
     if (has_err(d.err)) return;
+    constexpr uint32_t kChunk = choice_d_chunk(ND);
+    using Stage = ChoiceStageD<ND, kChunk>;
     uint64_t *W = reinterpret_cast<uint64_t *>(smem);
     uint64_t *PT = W + d.M;
-    uint32_t live_bits = 0;
+    Stage *const SB = reinterpret_cast<Stage *>(PT + d.M);
+    const int lane = threadIdx.x & 31;
+    uint32_t live_bits = 0;   // bit k: instance threadIdx.x + k * blockDim.x is live (M <= 32 * 288)
     for (uint32_t i = threadIdx.x, k = 0; i < d.M; i += blockDim.x, ++k) {
         W[i] = d.W[i];
         PT[i] = d.q_tail[i];
         live_bits |= uint32_t(d.inst_state[i] == 1) << k;
     }
-    __syncthreads();
-    const uint32_t nd = d.nd;
     const uint64_t cost = d.cost, slo = d.slo;
-    uint64_t tokens = 0, hits = 0, sw = 0, est = 0;
-    if (threadIdx.x == 0) {
-        for (uint32_t r = 0; r < n; ++r) {
-            const uint32_t *c = d.rd_cand + uint64_t(r) * nd, *h = d.rd_hit + uint64_t(r) * nd;
-            const uint32_t L = d.r_L[r];
-            uint32_t hmax = 0, nmax = 0, a = 0;
-            for (uint32_t f = 0; f < nd; ++f) hmax = max(hmax, h[f]);
-            bool all_over = true, first = true;
-            for (uint32_t f = 0; f < nd; ++f) {
-                const uint64_t t = W[c[f]] + cost * (L - h[f]);
-                o.ttft[uint64_t(r) * nd + f] = t;
-                all_over = all_over && t > slo;
-                if (h[f] == hmax) {
-                    ++nmax;
-                    if (first || W[c[f]] < W[c[a]]) a = f;
-                    first = false;
-                }
+    MetricSums ms{0, 0, 0, 0};
+
+    auto stage = [&](uint32_t buf, uint32_t k, uint32_t m, uint32_t base) {
+        if ((k & ~31u) >= m) return;   // no request in this window
+        Stage &S = SB[buf];
+        const bool valid = k < m;
+        uint32_t ids[(ND + 1) / 2];
+#pragma unroll
+        for (uint32_t x = 0; x < (ND + 1) / 2; ++x) ids[x] = 0xFFFFFFFFu;
+        if (valid) {
+            const uint32_t r = base + k, L = d.r_L[r];
+            const uint32_t *c = d.rd_cand + uint64_t(r) * ND, *h = d.rd_hit + uint64_t(r) * ND;
+            uint32_t cf[ND], hf[ND], hmax = 0;
+#pragma unroll
+            for (uint32_t f = 0; f < ND; ++f) {
+                cf[f] = c[f];
+                hf[f] = h[f];
+                hmax = max(hmax, hf[f]);
             }
-            uint32_t pick = a;
-            const bool over = nmax < nd && W[c[a]] + cost * (L - h[a]) > slo;
-            if (over)
-                for (uint32_t f = 0; f < nd; ++f)
-                    if (W[c[f]] < W[c[pick]]) pick = f;
-            const uint32_t ch = c[pick];
-            const uint64_t u = cost * (L - h[pick]);
-            o.chosen[r] = ch;
-            o.switched[r] = over;
-            for (uint32_t f = 0; f < nd; ++f) {
-                o.cand[uint64_t(r) * nd + f] = c[f];
-                o.hit[uint64_t(r) * nd + f] = h[f];
+            uint32_t most = 0;
+#pragma unroll
+            for (uint32_t f = 0; f < ND; ++f) {
+                S.c[f][k] = (uint16_t)cf[f];
+                S.u[f][k] = cost * (L - hf[f]);
+                most |= uint32_t(hf[f] == hmax) << f;
+                ids[f / 2] = f & 1 ? (ids[f / 2] & 0xFFFFu) | cf[f] << 16 : 0xFFFF0000u | cf[f];
+                o.cand[uint64_t(r) * ND + f] = cf[f];
+                o.hit[uint64_t(r) * ND + f] = hf[f];
             }
-            if (all_over) d.info->both_over = 1;
-            const uint64_t Pold = PT[ch];
-            W[ch] += u;
-            PT[ch] = Pold + (uint64_t(d.r_nblk[r]) << 32) + 1;
-            d.r_final[r] = ch;
-            d.r_touchoff[r] = Pold >> 32;   // offset among this batch's records of ch
-            tokens += L;
-            hits += h[pick];
-            sw += over;
-            est += W[ch] <= slo;
-            const uint32_t slot = (uint32_t)Pold;
-            if (slot - d.q_head[ch] >= d.Q) {
-                set_err(d.err, DM_ERR_CAPACITY);
-                continue;
-            }
-            QEntry e;
-            e.seq = seq0 + r;
-            e.work = e.remaining = u;
-            e.L = L;
-            e.c1 = c[0];
-            e.c2 = nd > 1 ? c[1] : c[0];
-            e.h1 = h[0];
-            e.h2 = nd > 1 ? h[1] : h[0];
-            e.moved = 0;
-            e.arrival = t_batch;
-            e.koff = 0;
-            DM_CHECK(ch < d.M, d.err);
-            d.q[uint64_t(ch) * d.Q + (slot & (d.Q - 1))] = e;
+            S.most[k] = (uint8_t)most;
         }
-    }
+        uint32_t nlev;
+        const uint32_t lev = window_levels<(ND + 1) / 2>(ids, valid, lane, nlev);
+        S.lev[k] = valid ? (uint8_t)lev : kNoLevel;
+        if (lane == 0) S.nlev[k / 32] = nlev;
+    };
+
+    auto decide = [&](uint32_t buf, uint32_t m) {
+        Stage &S = SB[buf];
+        volatile uint64_t *const Wv = W;
+        for (uint32_t w0 = 0; w0 < m; w0 += 32) {
+            const uint32_t k = w0 + lane;
+            const uint32_t mine = S.lev[k], nlev = S.nlev[w0 / 32], most = S.most[k];
+            uint32_t c[ND];
+            uint64_t u[ND], oW[ND];
+            uint32_t opick = 0;
+            bool oover = false;
+#pragma unroll
+            for (uint32_t f = 0; f < ND; ++f) {
+                c[f] = mine != kNoLevel ? S.c[f][k] : 0;
+                u[f] = S.u[f][k];   // past the batch's end: unused
+                oW[f] = 0;
+            }
+            for (uint32_t l = 0; l < nlev; ++l) {
+                uint64_t w[ND];
+#pragma unroll
+                for (uint32_t f = 0; f < ND; ++f) w[f] = Wv[c[f]];
+                // a: the least loaded of those with the most hit tokens (tie: the earlier ring)
+                uint64_t wa = ~0ull, ua = 0, wm = ~0ull, um = 0;
+                uint32_t a = ND, cm = 0, fm = 0, ca = 0;
+#pragma unroll
+                for (uint32_t f = 0; f < ND; ++f) {
+                    const bool ta = ((most >> f) & 1u) && (a == ND || w[f] < wa);
+                    wa = ta ? w[f] : wa;
+                    ua = ta ? u[f] : ua;
+                    ca = ta ? c[f] : ca;
+                    a = ta ? f : a;
+                    const bool tm = f == 0 || w[f] < wm;
+                    wm = tm ? w[f] : wm;
+                    um = tm ? u[f] : um;
+                    cm = tm ? c[f] : cm;
+                    fm = tm ? f : fm;
+                }
+                // over: some candidate has fewer hits and a misses the SLO; then
+                // the least loaded of all (tie: a, then the earlier ring)
+                const bool over = most != (1u << ND) - 1u && wa + ua > slo;
+                const bool mv = over && wm < wa;
+                if (mine == l) {
+                    Wv[mv ? cm : ca] = mv ? wm + um : wa + ua;
+#pragma unroll
+                    for (uint32_t f = 0; f < ND; ++f) oW[f] = w[f];
+                    opick = mv ? fm : a;
+                    oover = over;
+                }
+                __syncwarp();
+            }
+#pragma unroll
+            for (uint32_t f = 0; f < ND; ++f) S.Wf[f][k] = oW[f];
+            S.pick[k] = (uint8_t)opick;
+            S.over[k] = oover;
+        }
+    };
+
+    auto emit = [&](uint32_t buf, uint32_t k, uint32_t m, uint32_t base) {
+        const Stage &S = SB[buf];
+        const bool valid = k < m;
+        const uint32_t r = base + k, pick = valid ? S.pick[k] : 0;
+        const uint32_t ch = valid ? S.c[pick][k] : 0;
+        const uint32_t nbr = valid ? d.r_nblk[r] : 0;
+        const uint64_t pt = record_place<kChunk>(PT, ch, (uint64_t(nbr) << 32) + 1, valid, k / 32, (m + 31) / 32,
+                                                 lane);
+        if (!valid) return;
+        bool all_over = true;
+#pragma unroll
+        for (uint32_t f = 0; f < ND; ++f) {
+            const uint64_t t = S.Wf[f][k] + S.u[f][k];
+            o.ttft[uint64_t(r) * ND + f] = t;
+            all_over = all_over && t > slo;
+        }
+        if (all_over) d.info->both_over = 1;
+        o.chosen[r] = ch;
+        o.switched[r] = S.over[k];
+        d.r_final[r] = ch;
+        d.r_touchoff[r] = pt >> 32;   // offset among this batch's records of ch
+        const uint32_t L = d.r_L[r];
+        const uint32_t *h = d.rd_hit + uint64_t(r) * ND;
+        ms.tokens += L;
+        ms.hits += h[pick];
+        ms.sw += S.over[k];
+        ms.est += S.Wf[pick][k] + S.u[pick][k] <= slo;
+        const uint32_t slot = (uint32_t)pt;
+        if (slot - d.q_head[ch] >= d.Q) {
+            set_err(d.err, DM_ERR_CAPACITY);
+            return;
+        }
+        QEntry e;
+        e.seq = seq0 + r;
+        e.work = e.remaining = S.u[pick][k];
+        e.L = L;
+        e.c1 = S.c[0][k];
+        e.c2 = S.c[ND > 1 ? 1 : 0][k];
+        e.h1 = h[0];
+        e.h2 = h[ND > 1 ? 1 : 0];
+        e.moved = 0;
+        e.arrival = t_batch;
+        e.koff = 0;
+        DM_CHECK(ch < d.M, d.err);
+        d.q[uint64_t(ch) * d.Q + (slot & (d.Q - 1))] = e;
+    };
+
     __syncthreads();
+    choice_pipeline<kChunk>(n, stage, decide, emit);
     unsigned __int128 S1 = 0, S2 = 0;
     uint32_t cnt = 0;
     for (uint32_t i = threadIdx.x, k = 0; i < d.M; i += blockDim.x, ++k) {
@@ -768,20 +969,37 @@ __global__ void __launch_bounds__(1024) k_choice_d(DevState d, dm_route_out_d o,
         }
     }
     if (threadIdx.x == 0) d.info->final_dirty = 0;
-    finish_metrics(d, n, MetricSums{tokens, hits, sw, est}, S1, S2, cnt);
+    finish_metrics(d, n, ms, S1, S2, cnt);
+}
+
+template <uint32_t ND>
+static cudaError_t launch_choice_d(const DevState &d, const dm_route_out_d &o, uint32_t n, uint64_t seq0,
+                                   uint64_t t_batch, cudaStream_t st) {
+    constexpr uint32_t kChunk = choice_d_chunk(ND);
+    const size_t smem = size_t(d.M) * 16 + 3 * sizeof(ChoiceStageD<ND, kChunk>);
+    static size_t configured = 0;
+    if (smem > configured) {
+        DM_TRY(cudaFuncSetAttribute(k_choice_d<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        configured = smem;
+    }
+    return launch_pdl(k_choice_d<ND>, 1, Pipe<kChunk>::kThreads, smem, st, d, o, n, seq0, t_batch);
 }
 
 cudaError_t launch_route_d(const DevState &d, const dm_batch &b, const dm_route_out_d &o, uint64_t seq0,
                            cudaStream_t st) {
     if (b.n == 0) return cudaSuccess;
     DM_TRY(launch_pdl(k_route_d, (b.n + 7) / 8, 256, 0, st, d, b.tokens, b.n));
-    const size_t smem = size_t(d.M) * 16;
-    static size_t configured = 0;
-    if (smem > configured) {
-        DM_TRY(cudaFuncSetAttribute(k_choice_d, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        configured = smem;
+    switch (d.nd) {
+        case 1: DM_TRY(launch_choice_d<1>(d, o, b.n, seq0, b.batch_time_us, st)); break;
+        case 2: DM_TRY(launch_choice_d<2>(d, o, b.n, seq0, b.batch_time_us, st)); break;
+        case 3: DM_TRY(launch_choice_d<3>(d, o, b.n, seq0, b.batch_time_us, st)); break;
+        case 4: DM_TRY(launch_choice_d<4>(d, o, b.n, seq0, b.batch_time_us, st)); break;
+        case 5: DM_TRY(launch_choice_d<5>(d, o, b.n, seq0, b.batch_time_us, st)); break;
+        case 6: DM_TRY(launch_choice_d<6>(d, o, b.n, seq0, b.batch_time_us, st)); break;
+        case 7: DM_TRY(launch_choice_d<7>(d, o, b.n, seq0, b.batch_time_us, st)); break;
+        case 8: DM_TRY(launch_choice_d<8>(d, o, b.n, seq0, b.batch_time_us, st)); break;
+        default: return cudaErrorInvalidValue;
     }
-    DM_TRY(launch_pdl(k_choice_d, 1, 1024, smem, st, d, o, b.n, seq0, b.batch_time_us));
     return cudaGetLastError();
 }
 
