@@ -405,7 +405,9 @@ dm_status dm_create(const dm_config *cfg, dm_handle **out) {
     A(dalloc(h, &d.seg_pub, d.max_segs));
     A(dalloc(h, &d.r_m1, c.max_batch));
     A(dalloc(h, &d.r_m2, c.max_batch));
-    A(dalloc(h, &d.fix_list, c.max_batch));   // every route task at most once
+    A(dalloc(h, &d.r_tail, c.max_batch));
+    A(dalloc(h, &d.r_tcarry, c.max_batch));
+    A(dalloc(h, &d.fix_list, 2ull * c.max_batch));   // every route task and every tail task at most once
     A(dalloc(h, &d.defer, d.max_segs * dm::kSegBlocks));
     // two sets of batch scratch: routing and dm_hash_prompts
     for (DevState *x : {&h->d, &h->dh}) {

@@ -264,8 +264,10 @@ cudaError_t launch_hash(const DevState &d, const dm_batch &b, int grid, cudaStre
 //     resident on c_f and the first miss is block 64 j_f or lies in segment
 //     j_f - 1, which the route task probes (keys from the segment's stored
 //     prefix values when they check against its record, else hashed again
-//     from the tokens).  When every head segment's first block is resident
-//     the run may go on past the head: it hashes on from there.
+//     from the tokens).  When every head segment is resident the run may
+//     go on past the head: a counter per request collects its tail segments
+//     and this finding, and whoever completes it has the run settled from
+//     the stored prefix values (tail_task).
 // A route task whose head is not published yet goes back on the queue;
 // after kRetries tries it moves to a list that the kernel's last CTA to
 // finish works off, when everything is published.  Nothing waits on a warp
@@ -386,32 +388,113 @@ __device__ __noinline__ void head_seg_keys(const DevState &d, const uint32_t *to
 }
 
 // The run past the head, on the candidates whose first miss is still
-// kNoMiss (every head block resident there): hashes the prompt on from
-// segment j0 (f1 only, from carry `carry`) and probes segment by segment
-// until each run ends.  Updates m1 and m2 on every lane (kNoMiss: the whole
-// prompt is resident).  Whole warp; not inlined (rare: a cached run longer
-// than the head).
-template <int U>
-__device__ __noinline__ void run_on(const DevState &d, const uint32_t *tokens, uint64_t pol, uint32_t r,
-                                    uint32_t nblk, uint32_t j0, uint64_t carry, const RouteView &rv, int lane,
-                                    uint32_t &m1, uint32_t &m2) {
-    const HashLane<U> hl(d, lane);
-    const uint4 *tok4 = reinterpret_cast<const uint4 *>(tokens + d.r_tokoff[r]);
+// kNoMiss (every head block resident there), once every segment of the
+// request is hashed: the tails' first blocks are tested 128 at a time (keys
+// from the stored prefix values and totals), then the one segment that holds
+// the run's end, as for the head.  Writes r_m1 and r_m2 (kNoMiss: the whole
+// prompt is resident).  Whole warp; not inlined (a cached run longer than
+// the head).
+//
+// Three round trips for a 131,072-token prompt.  Hashing the prompt on from
+// its head, one segment per round trip, while the tokens were still being
+// hashed by the other warps took the kernel from 53 to 287 us when a few
+// prompts of a long-context batch were cached to their end, and to 254 us on
+// 64 follow-ups of 16k-114k cached tokens (GB300).
+constexpr uint32_t kTailVec = 4;
+__device__ __noinline__ void tail_task(const DevState &d, uint32_t r, int lane) {
+    const uint32_t nblk = d.r_nblk[r], s0 = d.r_segoff[r];
     const uint32_t nseg = (nblk + kSegBlocks - 1) / kSegBlocks;
+    const uint64_t *pl = d.plocal + d.r_blkoff[r];
+    const uint32_t ca = __ldcg(d.r_c1 + r), cb = __ldcg(d.r_c2 + r);
+    const RouteView rv{d.table[ca], d.table[cb], d.log_front[ca], d.log_front[cb]};
     const uint64_t mask = d.S - 1;
-    for (uint32_t j = j0; j < nseg && (m1 == kNoMiss || m2 == kNoMiss); ++j) {
-        const uint32_t c0 = j * kSegBlocks, cn = min(kSegBlocks, nblk - c0);
-        uint64_t P[2], tot, s2u;
-        hash_segment<U, false, false>(hl, tok4 + uint64_t(c0) * d.B / 4, c0, cn, 0, lane, pol, P, tot, s2u,
-                                      nullptr);
-        const uint64_t key[2] = {cache_key(P[0] + carry, d.Sc), cache_key(P[1] + carry, d.Sc)};
-        uint32_t e1, e2;
-        probe_segment(key, c0, c0 + cn, m1 == kNoMiss, m2 == kNoMiss, rv, mask, d.err, d.loop_limit, lane, e1,
-                      e2);
-        if (m1 == kNoMiss) m1 = e1;
-        if (m2 == kNoMiss) m2 = e2;
-        carry += tot;
+    uint32_t m1 = __ldcg(d.r_m1 + r), m2 = __ldcg(d.r_m2 + r);
+    bool open1 = m1 == kNoMiss, open2 = m2 == kNoMiss;
+    uint64_t carry = __ldcg(d.r_tcarry + r);   // into segment j0
+    uint64_t before = 0;                       // into segment j0 - 1 (j0 > H)
+    for (uint32_t j0 = d.H; j0 < nseg && (open1 || open2); j0 += 32 * kTailVec) {
+        uint64_t tot[kTailVec], key[kTailVec], in[kTailVec];
+#pragma unroll
+        for (uint32_t q = 0; q < kTailVec; ++q) {
+            const uint32_t sg = j0 + 32 * q + lane;
+            tot[q] = sg < nseg ? __ldcg(d.seg_total + s0 + sg) : 0;
+            key[q] = sg < nseg ? __ldcg(pl + uint64_t(sg) * kSegBlocks) : 0;
+        }
+        uint64_t c = carry;
+#pragma unroll
+        for (uint32_t q = 0; q < kTailVec; ++q) {
+            const uint64_t inc = warp_incl_scan(tot[q], lane);
+            in[q] = c + inc - tot[q];
+            key[q] = cache_key(key[q] + in[q], d.Sc);
+            c += shfl_u64(inc, 31);
+        }
+        // first segment of this round whose first block is missing (nseg or
+        // the round's end: none)
+        const uint32_t end = min(nseg, j0 + 32 * kTailVec);
+#pragma unroll 1
+        for (int f = 0; f < 2; ++f) {
+            if (!(f ? open2 : open1)) continue;
+            const Slot *t = f ? rv.t2 : rv.t1;
+            const uint64_t front = f ? rv.f2 : rv.f1;
+            Slot sl[kTailVec];
+#pragma unroll
+            for (uint32_t q = 0; q < kTailVec; ++q)
+                sl[q] = j0 + 32 * q + lane < nseg ? load_slot(t + group_home(key[q], 0, mask)) : Slot{0, 0};
+            uint32_t jf = end;
+#pragma unroll
+            for (uint32_t q = 0; q < kTailVec; ++q) {
+                const uint32_t sg = j0 + 32 * q + lane;
+                const bool miss = sg < nseg && !resident_at(t, mask, key[q], group_home(key[q], 0, mask), front,
+                                                            sl[q], d.err, d.loop_limit);
+                const uint32_t bal = __ballot_sync(0xffffffffu, miss);
+                if (bal && jf == end) jf = j0 + 32 * q + __ffs(bal) - 1;
+            }
+            if (jf == end && end < nseg) continue;   // goes on in the next round
+            // the run ends in segment jf - 1 or at block 64 jf (past the
+            // last segment: the whole prompt); the head is resident
+            const uint32_t s = jf - 1;
+            uint32_t e1 = kNoMiss, e2 = kNoMiss;
+            if (s >= d.H) {
+                uint64_t cs = before;
+#pragma unroll
+                for (uint32_t q = 0; q < kTailVec; ++q) {
+                    const uint64_t x = shfl_u64(in[q], (s - j0) & 31);
+                    if (s >= j0 && (s - j0) / 32 == q) cs = x;
+                }
+                const uint32_t c0 = s * kSegBlocks, cn = min(kSegBlocks, nblk - c0);
+                const uint64_t P0 = (uint32_t)lane < cn ? __ldcg(pl + c0 + lane) : 0;
+                const uint64_t P1 = (uint32_t)lane + 32 < cn ? __ldcg(pl + c0 + lane + 32) : 0;
+                const uint64_t k2[2] = {cache_key(P0 + cs, d.Sc), cache_key(P1 + cs, d.Sc)};
+                probe_segment(k2, c0, c0 + cn, f == 0, f == 1, rv, mask, d.err, d.loop_limit, lane, e1, e2);
+            }
+            const uint32_t e = f ? e2 : e1;
+            const uint32_t m = e != kNoMiss ? e : (jf < nseg ? jf * kSegBlocks : kNoMiss);
+            if (f) {
+                m2 = m;
+                open2 = false;
+            } else {
+                m1 = m;
+                open1 = false;
+            }
+        }
+        before = shfl_u64(in[kTailVec - 1], 31);
+        carry = c;
     }
+    if (lane == 0) {
+        d.r_m1[r] = m1;
+        d.r_m2[r] = m2;
+    }
+}
+
+// `k` more of request r's tail parts are done (its tail segments hashed, and
+// its route task when that found a run that goes on past the head): true in
+// the one caller that completes them.  The caller's writes before this are
+// visible to the warp that then runs the tail task.  One thread.
+__device__ __forceinline__ bool tail_done(const DevState &d, uint32_t r, uint32_t nseg, uint32_t k) {
+    __threadfence();
+    const bool all = atomicAdd(d.r_tail + r, k) + k == nseg - d.H + 1;
+    if (all) __threadfence();
+    return all;
 }
 
 // The route task of request r.  Returns false, changing nothing, when a head
@@ -478,15 +561,24 @@ __device__ __noinline__ bool route_task(const DevState &d, const uint32_t *token
         if (do1) m1 = e1 != kNoMiss ? e1 : (j1 < hs ? j1 * kSegBlocks : kNoMiss);
         if (do2) m2 = e2 != kNoMiss ? e2 : (j2 < hs ? j2 * kSegBlocks : kNoMiss);
     }
-    // every head block resident on a candidate: its run may go on past the head
-    if ((m1 == kNoMiss || m2 == kNoMiss) && hs < nseg)
-        run_on<U>(d, tokens, pol, r, nblk, hs, shfl_u64(inc1, hs - 1), rv, lane, m1, m2);
+    // every head block resident on a candidate: its run may go on past the
+    // head, which is settled once all tail segments are hashed
+    const bool past = (m1 == kNoMiss || m2 == kNoMiss) && hs < nseg;
+    bool tail = false;
     if (lane == 0) {
         d.r_K[r] = K;
         d.r_c1[r] = a;
         d.r_c2[r] = b;
         d.r_m1[r] = m1;
         d.r_m2[r] = m2;
+    }
+    if (past) {
+        const uint64_t hc = shfl_u64(inc1, hs - 1);
+        if (lane == 0) {
+            d.r_tcarry[r] = hc;
+            tail = tail_done(d, r, nseg, 1);
+        }
+        if (__shfl_sync(0xffffffffu, tail, 0)) tail_task(d, r, lane);
     }
     return true;
 }
@@ -565,6 +657,7 @@ struct CtaQueue {
     uint32_t busy;        // warps inside a route task
 };
 
+constexpr uint64_t kTailEntry = 1ull << 63;
 __device__ __forceinline__ uint64_t qentry(uint32_t r, uint32_t tries) {
     return uint64_t(r) | uint64_t(tries + 1) << 32;   // never 0
 }
@@ -772,6 +865,13 @@ __global__ void __launch_bounds__(HP<U>::kThreads, kMinBlocks) k_hash_probe(cons
         // m[s]: the warp's k-th task + s; the copies of m[0 .. S-2] are
         // issued, m[S-1] is looked up and issued next
         TaskMeta m[S];
+        // the request whose tail segments this warp is hashing (kNoTask:
+        // none), its segments in all, and how many it has hashed here
+        uint32_t tr = kNoTask, tns = 0, tcnt = 0;
+        auto tail_flush = [&] {
+            __syncwarp();
+            if (lane == 0 && tr != kNoTask && tail_done(d, tr, tns, tcnt)) q_push(q, d, uint64_t(tr) | kTailEntry);
+        };
 #pragma unroll
         for (int s = 0; s < S; ++s) {
             m[s] = cur_t.next(d, lane);
@@ -826,12 +926,21 @@ __global__ void __launch_bounds__(HP<U>::kThreads, kMinBlocks) k_hash_probe(cons
                         seg_pub_write(d.seg_pub + seg, E, tot1, sum2, pf, kk < kSegBlocks ? pk : 0, px);
                         if (cur.j + 1 == hs) q_push(q, d, qentry(cur.r, 0));   // the request's route task
                     }
+                } else {
+                    if (cur.r != tr) {
+                        tail_flush();
+                        tr = cur.r;
+                        tns = (cur.nblk + kSegBlocks - 1) / kSegBlocks;
+                        tcnt = 0;
+                    }
+                    ++tcnt;
                 }
             }
 #pragma unroll
             for (int s = 0; s + 1 < S; ++s) m[s] = m[s + 1];
             m[S - 1] = mn;
         }
+        tail_flush();
         // copies still in flight (only after a timeout): let them land
         for (uint32_t s = 0; s < (uint32_t)S; ++s)
             if ((pend >> s) & 1) mbar_wait(bar + s, (par >> s) & 1, kWaitLimit);
@@ -863,7 +972,9 @@ __global__ void __launch_bounds__(HP<U>::kThreads, kMinBlocks) k_hash_probe(cons
             }
             idle = 0;
             const uint32_t r = (uint32_t)e, tries = (uint32_t)(e >> 32) - 1;
-            const bool done = route_task<U, kAdapt>(d, tokens, E, pol, r, lane);
+            bool done = true;
+            if (e & kTailEntry) tail_task(d, r, lane);
+            else done = route_task<U, kAdapt>(d, tokens, E, pol, r, lane);
             if (lane == 0) {
                 if (!done) {
                     // a head segment hashed elsewhere not published yet: back on the queue
@@ -888,9 +999,12 @@ __global__ void __launch_bounds__(HP<U>::kThreads, kMinBlocks) k_hash_probe(cons
     __threadfence();
     const uint32_t nf = *(volatile uint32_t *)&d.info->fix_n;
     const uint32_t nw = blockDim.x >> 5;
-    for (uint32_t i = wid; i < nf; i += nw)
-        if (!route_task<U, kAdapt>(d, tokens, E, pol, (uint32_t)d.fix_list[i], lane) && lane == 0)
+    for (uint32_t i = wid; i < nf; i += nw) {
+        const uint64_t e = __ldcg(d.fix_list + i);
+        if (e & kTailEntry) tail_task(d, (uint32_t)e, lane);
+        else if (!route_task<U, kAdapt>(d, tokens, E, pol, (uint32_t)e, lane) && lane == 0)
             set_err(d.err, DM_ERR_TIMEOUT);   // cannot happen: everything is published by now
+    }
 }
 
 // Launch shape of the routing kernel per device and block size: its

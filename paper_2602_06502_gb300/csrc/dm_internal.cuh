@@ -252,6 +252,11 @@ struct DevState {
     // to the kernel's last CTA
     SegPub *seg_pub;
     uint32_t *r_m1, *r_m2;
+    // a request longer than its head: tail segments hashed so far, plus 1
+    // once its route task found a run that may go on past the head, and the
+    // f1 carry into the tail it left for that
+    uint32_t *r_tail;
+    uint64_t *r_tcarry;
     // DM_REBALANCE_FRESH_HITS (KQ = 0 otherwise): per instance a ring of KQ
     // block keys of its queued requests (instance i's at kring + i KQ), with
     // monotonic head and tail positions; per request of the pending batch
@@ -259,7 +264,7 @@ struct DevState {
     uint64_t KQ;
     uint64_t *kring, *kr_head, *kr_tail, *r_koff;
     uint32_t *rb_hq;                // rebalance scratch: a candidate's hit on its other candidate, per queue slot
-    uint64_t *fix_list;             // queue entries of route tasks (request, tries)
+    uint64_t *fix_list;             // queue entries of route and tail tasks
     uint64_t *seg_total, *seg_carry, *plocal;
     uint64_t *p2local;              // adaptive only: per block < Kf2, in-segment prefix of its f2 digests
     uint32_t *r_K;                  // per request: the hash prefix length it was routed with

@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(1024) k_setup(DevState d, const uint64_t *off,
                 const uint32_t ho = (uint32_t)e1, co = (uint32_t)(e1 >> 32), to = (uint32_t)(carry[2] + ex[2]);
                 d.r_hoff[r] = ho;
                 d.r_toff[r] = to;
+                d.r_tail[r] = 0;
                 d.r_segoff[r] = co + ho + to;
             } else {
                 d.r_segoff[r] = (uint32_t)(carry[1] + ex[1]);
