@@ -542,9 +542,10 @@ __device__ __noinline__ bool route_task(const DevState &d, const uint32_t *token
         miss2 = !resident_at(rv.t2, mask, key, home, rv.f2, load_slot(rv.t2 + home), d.err, d.loop_limit);
     }
     // j_f: the first head segment whose first block is missing on c_f (hs:
-    // none; lanes >= hs count as missing)
-    const uint32_t j1 = __ffs(__ballot_sync(0xffffffffu, miss1)) - 1;
-    const uint32_t j2 = __ffs(__ballot_sync(0xffffffffu, miss2)) - 1;
+    // none; lanes >= hs count as missing, and a head of 32 segments has no
+    // such lane)
+    const uint32_t b1 = __ballot_sync(0xffffffffu, miss1), b2 = __ballot_sync(0xffffffffu, miss2);
+    const uint32_t j1 = b1 ? __ffs(b1) - 1 : 32u, j2 = b2 ? __ffs(b2) - 1 : 32u;
     // the run on c_f ends in segment j_f - 1 or at block 64 j_f (when j_f <
     // hs); probe that segment, once for both candidates when they agree
     uint32_t m1 = j1 == 0 ? 0 : kNoMiss, m2 = j2 == 0 ? 0 : kNoMiss;
