@@ -116,15 +116,15 @@ __device__ void finish_metrics(const DevState &d, uint32_t n, MetricSums ms, uns
 // choice, one thread from global memory before: 5,360 and 577 us (d = 4).
 constexpr uint8_t kNoLevel = 255;
 
-template <uint32_t kChunk>
+template <uint32_t kChunk, uint32_t kStageThreads = kChunk>
 struct Pipe {
-    static constexpr uint32_t kWindows = kChunk / 32;
-    static constexpr uint32_t kThreads = 32 + 2 * kChunk;   // warp 0, the emitting warps, the staging warps
+    static constexpr uint32_t kThreads = 32 + kChunk + kStageThreads;   // warp 0, the emitting and staging warps
 };
 
 // stage(buffer, k, m, base), decide(buffer, m), emit(buffer, k, m, base): k
-// this thread's request of the chunk (whole windows call; k >= m past the
-// batch's end), m its requests, base its first request.
+// the thread's number among its role's (an emitting thread's request of the
+// chunk; whole windows call, k >= m past the batch's end), m the chunk's
+// requests, base its first request.
 template <uint32_t kChunk, class StageF, class DecideF, class EmitF>
 __device__ __forceinline__ void choice_pipeline(uint32_t n, StageF stage, DecideF decide, EmitF emit) {
     const uint32_t nc = (n + kChunk - 1) / kChunk, tid = threadIdx.x;
@@ -414,58 +414,340 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads) k_choice(DevStat
 // Cluster-wide rules.
 
 // Hit tokens of every request on every live instance (0 elsewhere), against
-// the index as of the start of the batch: one warp per (request, instance)
-// pair, grid-stride.  The first step tests 32 blocks (most instances miss
-// block 0), later steps 128 (4 independent lookups per lane); a slot that
-// holds the key or is empty settles the lookup at its home slot, anything
-// else takes the full probe order.
+// the index as of the start of the batch: a warp per request and 32
+// instances, a lane per instance.  The keys resident on an instance are
+// closed under prefixes (see the routing kernel), so a lane tests block 0
+// and, where that is resident (most instances miss it), finds the run's end
+// by bisection; lanes that probe the same block read the same prefix value.
+// Bound by random 16-byte index reads (one to ten a pair).  4,096 agent
+// prompts x 64 instances, GB300: 822 us with a warp per pair testing 32, then
+// 128 blocks a round; 183 us so.
 constexpr int kAllBlock = 256;
 
 __global__ void __launch_bounds__(kAllBlock) k_probe_all(DevState d, uint32_t n) {
     pdl_enter();
     if (has_err(d.err)) return;
     const int lane = threadIdx.x & 31;
-    const uint64_t nw = uint64_t(gridDim.x) * (kAllBlock / 32);
-    const uint64_t total = uint64_t(n) * d.M;
+    const uint32_t groups = (d.M + 31) / 32;
+    const uint64_t total = uint64_t(n) * groups, nw = uint64_t(gridDim.x) * (kAllBlock / 32);
     const uint64_t mask = d.S - 1;
     for (uint64_t p = (uint64_t(blockIdx.x) * kAllBlock + threadIdx.x) / 32; p < total; p += nw) {
-        const uint32_t r = (uint32_t)(p / d.M), i = (uint32_t)(p - uint64_t(r) * d.M);
+        const uint32_t r = (uint32_t)(p / groups), i = (uint32_t)(p - uint64_t(r) * groups) * 32 + lane;
+        if (i >= d.M) continue;
         uint32_t h = 0;
         if (d.inst_state[i] == 1) {
             const uint32_t nblk = d.r_nblk[r], s0 = d.r_segoff[r];
-            const uint64_t bo = d.r_blkoff[r];
+            const uint64_t *pl = d.plocal + d.r_blkoff[r];
             const Slot *t = d.table[i];
             const uint64_t front = d.log_front[i];
-            for (uint32_t base = 0, step = 1;; base += 32 * step, step = 4) {
-                uint64_t key[4], home[4];
-                Slot sl[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint32_t b = base + 32 * j + lane;   // windows of 32 keep the groups whole
-                    const bool inb = j < (int)step && b < nblk;
-                    key[j] = inb ? cache_key(d.plocal[bo + b] + d.seg_carry[s0 + b / kSegBlocks], d.Sc) : 0;
-                    home[j] = group_home(group_anchor(key[j], lane), b, mask);
-                    if (inb) sl[j] = load_slot(t + home[j]);
+            auto resident = [&](uint32_t b) {
+                const uint64_t carry = d.seg_carry[s0 + b / kSegBlocks];
+                const uint64_t key = cache_key(pl[b] + carry, d.Sc);
+                const uint64_t anchor = cache_key(pl[b & ~(kGroup - 1)] + carry, d.Sc);
+                const uint64_t home = group_home(anchor, b, mask);
+                return resident_at(t, mask, key, home, front, load_slot(t + home), d.err, d.loop_limit);
+            };
+            if (resident(0)) {
+                uint32_t lo = 0, hi = nblk;   // block lo is resident; hi is not, or the prompt's end
+                while (hi - lo > 1) {
+                    const uint32_t mid = lo + (hi - lo) / 2;
+                    if (resident(mid)) lo = mid;
+                    else hi = mid;
                 }
-                uint32_t miss_at = 0xFFFFFFFFu;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const bool res = key[j] != 0 && resident_at(t, mask, key[j], home[j], front, sl[j], d.err, d.loop_limit);
-                    const uint32_t m = __ballot_sync(0xffffffffu, !res);
-                    if (j < (int)step && m && miss_at == 0xFFFFFFFFu) miss_at = base + 32 * j + __ffs(m) - 1;
-                }
-                if (miss_at != 0xFFFFFFFFu) {
-                    h = miss_at;
-                    break;
-                }
+                h = hi;
             }
         }
-        if (lane == 0) d.h_all[p] = h * d.B;
+        d.h_all[uint64_t(r) * d.M + i] = h * d.B;
     }
 }
 
-// k_choice_global: W and PT per instance and the live ids, then, for a
-// chunk of `cap` requests, their per-request fields, their decisions and
+// ---------------------------------------------------------------------------
+// The cluster-wide choice over up to 512 instances, pipelined like the pair
+// choice.  Every request depends on the one before it, so the chain is the
+// argmin over the instances: their loads stay in the deciding warp's
+// registers (lane l holds the live ids of list indices J l .. J l + J - 1),
+// as 32-bit offsets from the smallest load, and one request is J compares, a
+// 32-bit minimum over the warp, a vote, and an add in the winning lane.  The
+// lowest lane with the smallest key holds the lowest id.  A chunk whose
+// loads and work do not fit 31 bits is decided in 64 bits instead.  The hits
+// come into shared memory a chunk ahead.
+// 4,096 agent prompts on 64 instances, min TTFT, GB300: 1,678 us with 64-bit
+// keys and loads in shared memory, three reductions a request, and staging
+// and emission between the chunks; 922 us so.
+constexpr uint32_t kGlobalStageThreads = 256;
+template <uint32_t J>
+struct GlobalPipe {
+    static constexpr uint32_t kChunk = J <= 8 ? 64 : 32;   // three buffers of hits fit at 512 instances
+    static constexpr uint32_t kThreads = Pipe<kChunk, kGlobalStageThreads>::kThreads;
+    struct Stage {
+        uint32_t hit[kChunk][32 * J];
+        uint64_t cl[kChunk];                    // cost x L
+        uint64_t t[2][kChunk], wch[kChunk];     // loads of c1 and c2 before, of the choice after
+        uint32_t ci[2][kChunk], hmax[kChunk];   // list indices of c1, c2; 0xFFFFFFFF hmax: no affinity
+        uint32_t ch[kChunk];                    // list index chosen
+    };
+    static size_t smem(uint32_t M) { return 32 * J * 20 + (size_t(M) * 2 + 15) / 16 * 16 + 3 * sizeof(Stage); }
+};
+
+template <uint32_t J>
+__global__ void __launch_bounds__(GlobalPipe<J>::kThreads) k_choice_all(DevState d, dm_route_out o, uint32_t n,
+                                                                        uint64_t seq0, uint64_t t_batch) {
+    pdl_enter();
+    using P = GlobalPipe<J>;
+    using Stage = typename P::Stage;
+    constexpr uint32_t kN = 32 * J, kChunk = P::kChunk;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint32_t s_wcnt[32];
+    if (has_err(d.err)) return;
+    // by list index: load, records << 32 | queue tail, id; by id: list index
+    uint64_t *W = reinterpret_cast<uint64_t *>(smem), *PT = W + kN;
+    uint32_t *live = reinterpret_cast<uint32_t *>(PT + kN);
+    uint16_t *inv = reinterpret_cast<uint16_t *>(live + kN);
+    Stage *const SB = reinterpret_cast<Stage *>(smem + kN * 20 + (size_t(d.M) * 2 + 15) / 16 * 16);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t nl = 0;   // live ids in ascending order
+    for (uint32_t base = 0; base < d.M; base += blockDim.x) {
+        const uint32_t i = base + threadIdx.x;
+        const bool f = i < d.M && d.inst_state[i] == 1;
+        const uint32_t bal = __ballot_sync(0xffffffffu, f);
+        if (lane == 0) s_wcnt[wid] = __popc(bal);
+        __syncthreads();
+        uint32_t off = nl, tot = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+            off += w < wid ? s_wcnt[w] : 0;
+            tot += s_wcnt[w];
+        }
+        if (f) {
+            const uint32_t k = off + __popc(bal & ((1u << lane) - 1));
+            live[k] = i;
+            inv[i] = (uint16_t)k;
+            W[k] = d.W[i];
+            PT[k] = d.q_tail[i];
+        }
+        nl += tot;
+        __syncthreads();
+    }
+    if (nl == 0) {   // the host requires two
+        if (threadIdx.x == 0) set_err(d.err, DM_ERR_NO_INSTANCES);
+        return;
+    }
+    const uint64_t cost = d.cost, slo = d.slo;
+    const uint32_t rule = d.rule;
+    MetricSums ms{0, 0, 0, 0};
+
+    auto stage = [&](uint32_t buf, uint32_t k, uint32_t m, uint32_t base) {
+        Stage &S = SB[buf];
+        for (uint32_t rr = k >> 5; rr < m; rr += kGlobalStageThreads / 32) {   // a warp per request
+            const uint32_t r = base + rr, L = d.r_L[r];
+            const uint32_t *ha = d.h_all + uint64_t(r) * d.M;
+            uint32_t h[J], hmax = 0;
+#pragma unroll
+            for (uint32_t j = 0; j < J; ++j) {
+                const uint32_t x = j * 32 + lane;
+                h[j] = x < nl ? ha[live[x]] : 0;
+            }
+#pragma unroll
+            for (uint32_t j = 0; j < J; ++j) {
+                S.hit[rr][j * 32 + lane] = h[j];
+                hmax = max(hmax, h[j]);
+            }
+            hmax = __reduce_max_sync(0xffffffffu, hmax);
+            if (lane == 0) {
+                S.cl[rr] = cost * L;
+                S.hmax[rr] = rule == DM_RULE_PREBLE && 2ull * hmax > L ? hmax : 0xFFFFFFFFu;
+                S.ci[0][rr] = inv[d.r_c1[r]];
+                S.ci[1][rr] = inv[d.r_c2[r]];
+            }
+        }
+    };
+
+    auto decide = [&](uint32_t buf, uint32_t m) {
+        Stage &S = SB[buf];
+        volatile uint64_t *const Wv = W;
+        uint64_t w64[J], lo = ~0ull, hi = 0, work = 0;
+        bool small = true;   // cost x L of every request fits 31 bits
+#pragma unroll
+        for (uint32_t j = 0; j < J; ++j) {
+            const uint32_t x = lane * J + j;
+            w64[j] = x < nl ? W[x] : ~0ull;
+            if (x < nl) {
+                lo = min(lo, w64[j]);
+                hi = max(hi, w64[j]);
+            }
+        }
+        for (uint32_t rr = lane; rr < m; rr += 32) {
+            small &= S.cl[rr] < (1ull << 31);
+            work += S.cl[rr];
+        }
+#pragma unroll
+        for (int x = 16; x >= 1; x >>= 1) {
+            lo = min(lo, shfl_xor_u64(lo, x));
+            hi = max(hi, shfl_xor_u64(hi, x));
+            work += shfl_xor_u64(work, x);
+        }
+        small = __all_sync(0xffffffffu, small);
+        constexpr uint32_t kNever = 0x80000000u;   // above every key that may win
+        if (small && hi - lo < kNever && work < kNever - (hi - lo)) {
+            uint32_t w[J];
+#pragma unroll
+            for (uint32_t j = 0; j < J; ++j) w[j] = lane * J + j < nl ? (uint32_t)(w64[j] - lo) : 0xFFFFFFFFu;
+            const uint32_t c32 = (uint32_t)cost;
+            // each request's keys less the loads, read one request ahead
+            uint32_t u[J], add[J];
+            auto read = [&](uint32_t rr) {
+                const uint32_t cl = (uint32_t)S.cl[rr], hm = S.hmax[rr];
+#pragma unroll
+                for (uint32_t j = 0; j < J; ++j) {
+                    const uint32_t h = S.hit[rr][lane * J + j];
+                    u[j] = cl - c32 * h;
+                    add[j] = rule == DM_RULE_LEAST_LOADED ? 0u : hm == 0xFFFFFFFFu ? u[j] : h == hm ? 0u : kNever;
+                    if (lane * J + j >= nl) add[j] = 0;   // w stays above every key
+                }
+            };
+            read(0);
+            for (uint32_t rr = 0; rr < m; ++rr) {
+                const uint64_t wc = lane < 2 ? Wv[S.ci[lane & 1][rr]] : 0;   // as this request finds them
+                __syncwarp();
+                uint32_t bk = w[0] + add[0], bu = u[0], bj = 0, bw = w[0];
+#pragma unroll
+                for (uint32_t j = 1; j < J; ++j) {
+                    const uint32_t key = w[j] + add[j];
+                    const bool less = key < bk;
+                    bk = less ? key : bk;
+                    bu = less ? u[j] : bu;
+                    bw = less ? w[j] : bw;
+                    bj = less ? j : bj;
+                }
+                const uint32_t kmin = __reduce_min_sync(0xffffffffu, bk);
+                const uint32_t eq = __ballot_sync(0xffffffffu, bk == kmin);
+                const bool win = bk == kmin && (eq & ((1u << lane) - 1u)) == 0;
+                const uint32_t nw = bw + bu;
+#pragma unroll
+                for (uint32_t j = 0; j < J; ++j) w[j] = win && bj == j ? nw : w[j];
+                if (win) {
+                    Wv[lane * J + bj] = lo + nw;
+                    S.wch[rr] = lo + nw;
+                    S.ch[rr] = lane * J + bj;
+                }
+                if (rr + 1 < m) read(rr + 1);
+                if (lane < 2) S.t[lane][rr] = wc;
+                __syncwarp();
+            }
+        } else {
+            for (uint32_t rr = 0; rr < m; ++rr) {
+                const uint64_t wc = lane < 2 ? Wv[S.ci[lane & 1][rr]] : 0;
+                const uint64_t cl = S.cl[rr];
+                const uint32_t hm = S.hmax[rr];
+                // smallest (key, list index): three 32-bit reductions give the exact pair
+                uint64_t bk = ~0ull;
+                uint32_t bx = 0xFFFFFFFFu;
+                for (uint32_t x = lane; x < nl; x += 32) {
+                    const uint32_t h = S.hit[rr][x];
+                    const uint64_t w = Wv[x];
+                    const uint64_t key = rule == DM_RULE_LEAST_LOADED ? w
+                                         : hm == 0xFFFFFFFFu          ? w + cl - cost * h
+                                         : h == hm                    ? w
+                                                                      : ~0ull;
+                    if (key < bk || bx == 0xFFFFFFFFu) {
+                        bk = key;
+                        bx = x;
+                    }
+                }
+                const uint32_t khi = __reduce_min_sync(0xffffffffu, (uint32_t)(bk >> 32));
+                const uint32_t klo =
+                    __reduce_min_sync(0xffffffffu, (uint32_t)(bk >> 32) == khi ? (uint32_t)bk : 0xFFFFFFFFu);
+                const uint32_t x =
+                    __reduce_min_sync(0xffffffffu, bk == ((uint64_t(khi) << 32) | klo) ? bx : 0xFFFFFFFFu);
+                __syncwarp();
+                if (lane == 0) {
+                    const uint64_t nw = Wv[x] + cl - cost * S.hit[rr][x];
+                    Wv[x] = nw;
+                    S.wch[rr] = nw;
+                    S.ch[rr] = x;
+                }
+                if (lane < 2) S.t[lane][rr] = wc;
+                __syncwarp();
+            }
+        }
+    };
+
+    auto emit = [&](uint32_t buf, uint32_t k, uint32_t m, uint32_t base) {
+        const Stage &S = SB[buf];
+        const bool valid = k < m;
+        const uint32_t r = base + k, x = valid ? S.ch[k] : 0;
+        const uint32_t nbr = valid ? d.r_nblk[r] : 0;
+        const uint64_t pt =
+            record_place<kChunk>(PT, x, (uint64_t(nbr) << 32) + 1, valid, k / 32, (m + 31) / 32, lane);
+        if (!valid) return;
+        const uint32_t ch = live[x], h = S.hit[k][x], L = d.r_L[r];
+        const uint32_t h1 = hit_tokens(d.r_m1[r], nbr, d.B), h2 = hit_tokens(d.r_m2[r], nbr, d.B);
+        const uint64_t t1 = S.t[0][k] + cost * (L - h1), t2 = S.t[1][k] + cost * (L - h2);
+        o.ttft1[r] = t1;
+        o.ttft2[r] = t2;
+        o.chosen[r] = ch;
+        o.switched[r] = 0;
+        d.r_final[r] = ch;
+        d.r_touchoff[r] = pt >> 32;
+        ms.tokens += L;
+        ms.hits += h;
+        ms.est += S.wch[k] <= slo;
+        if (t1 > slo && t2 > slo) d.info->both_over = 1;
+        const uint32_t slot = (uint32_t)pt;
+        if (slot - d.q_head[ch] >= d.Q) {
+            set_err(d.err, DM_ERR_CAPACITY);
+            return;
+        }
+        QEntry e;
+        e.seq = seq0 + r;
+        e.work = e.remaining = cost * (L - h);
+        e.L = L;
+        e.c1 = d.r_c1[r];
+        e.c2 = d.r_c2[r];
+        e.h1 = h1;
+        e.h2 = h2;
+        e.moved = 0;
+        e.arrival = t_batch;
+        e.koff = 0;
+        DM_CHECK(ch < d.M, d.err);
+        d.q[uint64_t(ch) * d.Q + (slot & (d.Q - 1))] = e;
+    };
+
+    choice_pipeline<kChunk>(n, stage, decide, emit);
+    unsigned __int128 S1 = 0, S2 = 0;
+    uint32_t cnt = 0;
+    for (uint32_t i = threadIdx.x; i < d.M; i += blockDim.x) {
+        if (d.inst_state[i] != 1) {
+            d.log_adv[i] = 0;
+            continue;
+        }
+        const uint32_t x = inv[i];
+        d.W[i] = W[x];
+        d.q_tail[i] = (uint32_t)PT[x];
+        d.log_adv[i] = PT[x] >> 32;
+        S1 += W[x];
+        S2 += (unsigned __int128)W[x] * W[x];
+        ++cnt;
+    }
+    if (threadIdx.x == 0) d.info->final_dirty = 0;
+    finish_metrics(d, n, ms, S1, S2, cnt);
+}
+
+template <uint32_t J>
+static cudaError_t launch_choice_all(const DevState &d, const dm_route_out &o, uint32_t n, uint64_t seq0,
+                                     uint64_t t_batch, cudaStream_t st) {
+    const size_t smem = GlobalPipe<J>::smem(d.M);
+    static size_t configured = 0;
+    if (smem > configured) {
+        DM_TRY(cudaFuncSetAttribute(k_choice_all<J>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        configured = smem;
+    }
+    return launch_pdl(k_choice_all<J>, 1, GlobalPipe<J>::kThreads, smem, st, d, o, n, seq0, t_batch);
+}
+
+// The same over any number of instances (max_instances above 512, where a
+// lane could not keep its instances' loads in registers nor the chunks'
+// hits fit three buffers).  k_choice_global: W and PT per instance and the
+// live ids, then, for a chunk of `cap` requests, their per-request fields, their decisions and
 // their hits on every live instance; cap is what the shared memory holds
 // (at most 1024).  The decisions are written out in parallel after each
 // chunk's sequential pass, which touches shared memory only.
@@ -637,23 +919,32 @@ cudaError_t launch_choice(const DevState &d, const dm_route_out &o, uint32_t n, 
                           cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     if (d.rule >= DM_RULE_LEAST_LOADED) {
-        // as much shared memory as the device allows, up to what 1024 requests need
-        static uint32_t smem_g = 0, smem_M = 0;
-        if (smem_M != d.M) {
-            int dev = 0, optin = 0;
-            cudaFuncAttributes fa{};
-            DM_TRY(cudaGetDevice(&dev));
-            DM_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-            DM_TRY(cudaFuncGetAttributes(&fa, k_choice_global));
-            const size_t want = global_stage_off(d.M) + size_t(kGlobalReqMax) * (kGlobalReqBytes + 4ull * d.M);
-            const size_t room = size_t(optin) - fa.sharedSizeBytes;
-            smem_g = (uint32_t)(want < room ? want : room);
-            DM_TRY(cudaFuncSetAttribute(k_choice_global, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_g));
-            smem_M = d.M;
-        }
         DM_TRY(launch_carries(d, o, n, st));
-        DM_TRY(launch_pdl(k_probe_all, full_grid(k_probe_all, kAllBlock), kAllBlock, 0, st, d, n));
-        DM_TRY(launch_pdl(k_choice_global, 1, 1024, smem_g, st, d, o, n, seq0, t_batch, smem_g));
+        const uint64_t warps = uint64_t(n) * ((d.M + 31) / 32);
+        const unsigned grid = (unsigned)std::min<uint64_t>((warps + kAllBlock / 32 - 1) / (kAllBlock / 32), 1u << 30);
+        DM_TRY(launch_pdl(k_probe_all, grid, kAllBlock, 0, st, d, n));
+        if (d.M <= 64) DM_TRY(launch_choice_all<2>(d, o, n, seq0, t_batch, st));
+        else if (d.M <= 128) DM_TRY(launch_choice_all<4>(d, o, n, seq0, t_batch, st));
+        else if (d.M <= 256) DM_TRY(launch_choice_all<8>(d, o, n, seq0, t_batch, st));
+        else if (d.M <= 512) DM_TRY(launch_choice_all<16>(d, o, n, seq0, t_batch, st));
+        else {
+            // as much shared memory as the device allows, up to what 1024 requests need
+            static uint32_t smem_g = 0, smem_M = 0;
+            if (smem_M != d.M) {
+                int dev = 0, optin = 0;
+                cudaFuncAttributes fa{};
+                DM_TRY(cudaGetDevice(&dev));
+                DM_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+                DM_TRY(cudaFuncGetAttributes(&fa, k_choice_global));
+                const size_t want = global_stage_off(d.M) + size_t(kGlobalReqMax) * (kGlobalReqBytes + 4ull * d.M);
+                const size_t room = size_t(optin) - fa.sharedSizeBytes;
+                smem_g = (uint32_t)(want < room ? want : room);
+                DM_TRY(cudaFuncSetAttribute(k_choice_global, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)smem_g));
+                smem_M = d.M;
+            }
+            DM_TRY(launch_pdl(k_choice_global, 1, 1024, smem_g, st, d, o, n, seq0, t_batch, smem_g));
+        }
         return cudaGetLastError();
     }
     const size_t smem = choice_smem(d.M);
