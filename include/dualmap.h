@@ -430,7 +430,7 @@ DM_API dm_status dm_hash_prompts(dm_handle *h, const dm_batch *batch, uint64_t *
                           uint64_t *key_off_dev, uint64_t *pos_dev);
 
 /* Limits of dm_hash_prompts_noalloc: requests per call, and full blocks per
- * call (total_tokens / block_tokens).  Its fixed scratch is about 2.2 MB. */
+ * call (total_tokens / block_tokens).  Its fixed scratch is about 1.5 MB. */
 #define DM_NOALLOC_MAX_REQUESTS 4096u
 #define DM_NOALLOC_MAX_BLOCKS 4194304ull
 
@@ -441,7 +441,7 @@ DM_API dm_status dm_hash_prompts(dm_handle *h, const dm_batch *batch, uint64_t *
  * device memory at the point they hash, for example a serving process whose
  * device memory is entirely owned by another allocator, or code on a path
  * where cudaMalloc's implicit synchronisation is not acceptable.
- * Working memory is one fixed array of about 2.2 MB inside the library, which
+ * Working memory is one fixed array of about 1.5 MB inside the library, which
  * every GPU that loads the library keeps until the process exits; keys_dev
  * (which must hold sum(n_blk) entries) doubles as working space.
  * Returns DM_ERR_CAPACITY without doing anything when n exceeds

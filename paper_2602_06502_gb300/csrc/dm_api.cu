@@ -920,7 +920,7 @@ dm_status dm_hash_prompts(dm_handle *h, const dm_batch *b, uint64_t *keys_dev, u
     if (b->n == 0) return DM_OK;
     cudaError_t e = dm::launch_setup(h->dh, *b, h->st);
     if (e == cudaSuccess) e = dm::launch_hash(h->dh, *b, h->hash_grid, h->st);
-    if (e == cudaSuccess) e = dm::launch_hash_keys(h->dh, b->n, keys_dev, key_off_dev, pos_dev, h->st);
+    if (e == cudaSuccess) e = dm::launch_hash_keys(h->dh, *b, keys_dev, key_off_dev, pos_dev, h->st);
     return map_cuda(h, e);
 }
 

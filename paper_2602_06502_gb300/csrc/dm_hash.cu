@@ -15,6 +15,7 @@
 // n_blk) blocks (Kf2 = K_route, or the longest adaptive prefix): segments
 // below K write the sum of their f2 digests and, with the adaptive length,
 // each block's in-segment f2 prefix value.
+#include <algorithm>
 #include <atomic>
 
 #include "dm_internal.cuh"
@@ -161,9 +162,25 @@ __device__ __forceinline__ void hash_segment(const HashLane<U> &hl, const uint4 
     hash_loaded<U, kF2, kP2>(hl, v, b0, nb, K, lane, P, tot1, sum2, p2out);
 }
 
-// Hashing only (dm_hash_prompts and the allocation-free variant): one warp
-// per segment in segment order; writes every block's local prefix value and
-// each segment's totals.
+// Request holding task x: the largest r < n with off[r] <= x (off:
+// exclusive offsets, nondecreasing, off[0] = 0).  The
+// whole warp narrows the range 32 ways per round trip (two for n <= 1024).
+__device__ __forceinline__ uint32_t find_req(const uint32_t *off, uint32_t n, uint32_t x, int lane) {
+    uint32_t lo = 0, len = n;   // the request lies in [lo, lo + len); off[lo] <= x
+    while (len > 1) {
+        const uint32_t step = (len + 31) / 32;
+        const bool le = (uint32_t)lane * step < len && __ldg(off + lo + lane * step) <= x;
+        const uint32_t k = 31 - __clz(__ballot_sync(0xffffffffu, le));   // lane 0 always holds
+        lo += k * step;
+        len = min(step, len - k * step);
+    }
+    return lo;
+}
+
+// Hashing only (dm_hash_prompts, its allocation-free variant, and routing
+// with d candidates): every warp takes a contiguous run of segments, finds
+// the first one's request once and follows the requests from there; writes
+// every block's local prefix value and each segment's totals and request.
 template <int U, bool kP2>
 __global__ void __launch_bounds__(256, 4) k_hash(DevState d, const uint32_t *__restrict__ tokens) {
     pdl_enter();
@@ -171,17 +188,26 @@ __global__ void __launch_bounds__(256, 4) k_hash(DevState d, const uint32_t *__r
     const int lane = threadIdx.x & 31;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
     const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t total_segs = d.info->total_segs;
+    const uint32_t total_segs = d.info->total_segs, n = d.info->n;
+    const uint32_t lo = uint32_t(uint64_t(total_segs) * gw / nwarps), hi = uint32_t(uint64_t(total_segs) * (gw + 1) / nwarps);
+    if (lo >= hi) return;
     const HashLane<U> hl(d, lane);
     const uint64_t pol = evict_first_policy();
-    for (uint32_t seg = gw; seg < total_segs; seg += nwarps) {
-        const uint32_t r = d.seg_req[seg];
-        const uint32_t j = seg - d.r_segoff[r];
-        const uint32_t nblk = d.r_nblk[r];
-        const uint32_t b0 = j * kSegBlocks;
+    uint32_t r = find_req(d.r_segoff, n, lo, lane);
+    uint32_t s0 = d.r_segoff[r], end = r + 1 < n ? d.r_segoff[r + 1] : total_segs, nblk = d.r_nblk[r];
+    uint64_t to = d.r_tokoff[r], bo = d.r_blkoff[r];
+    for (uint32_t seg = lo; seg < hi; ++seg) {
+        if (seg >= end) {   // every request has a segment
+            ++r;
+            s0 = end;
+            end = r + 1 < n ? d.r_segoff[r + 1] : total_segs;
+            nblk = d.r_nblk[r];
+            to = d.r_tokoff[r];
+            bo = d.r_blkoff[r];
+        }
+        const uint32_t b0 = (seg - s0) * kSegBlocks;
         const uint32_t nb = min(kSegBlocks, nblk - b0);
-        const uint4 *src4 = reinterpret_cast<const uint4 *>(tokens + d.r_tokoff[r] + uint64_t(b0) * d.B);
-        const uint64_t bo = d.r_blkoff[r];
+        const uint4 *src4 = reinterpret_cast<const uint4 *>(tokens + to + uint64_t(b0) * d.B);
         uint64_t P[2], tot1, sum2;
         hash_segment<U, true, kP2>(hl, src4, b0, nb, min(d.Kf2, nblk), lane, pol, P, tot1, sum2,
                                    kP2 ? d.p2local + bo + b0 : nullptr);
@@ -191,6 +217,7 @@ __global__ void __launch_bounds__(256, 4) k_hash(DevState d, const uint32_t *__r
         if (lane == 0) {
             d.seg_total[seg] = tot1;
             d.seg_total2[seg] = sum2;
+            d.seg_req[seg] = r;
         }
     }
 }
@@ -273,21 +300,6 @@ cudaError_t launch_hash(const DevState &d, const dm_batch &b, int grid, cudaStre
 // finish works off, when everything is published.  Nothing waits on a warp
 // of another CTA.  The segment carries of the whole batch, which the commit
 // needs, and the route outputs are produced by the choice kernel's launch.
-
-// Request holding task x of a part: the largest r < n with off[r] <= x
-// (off: exclusive offsets of that part, nondecreasing, off[0] = 0).  The
-// whole warp narrows the range 32 ways per round trip (two for n <= 1024).
-__device__ __forceinline__ uint32_t find_req(const uint32_t *off, uint32_t n, uint32_t x, int lane) {
-    uint32_t lo = 0, len = n;   // the request lies in [lo, lo + len); off[lo] <= x
-    while (len > 1) {
-        const uint32_t step = (len + 31) / 32;
-        const bool le = (uint32_t)lane * step < len && __ldg(off + lo + lane * step) <= x;
-        const uint32_t k = 31 - __clz(__ballot_sync(0xffffffffu, le));   // lane 0 always holds
-        lo += k * step;
-        len = min(step, len - k * step);
-    }
-    return lo;
-}
 
 // Loads through L2 (data written by other warps during this kernel).
 __device__ __forceinline__ void ld_cg2(const void *p, uint64_t &a, uint64_t &b) {
@@ -1130,33 +1142,102 @@ cudaError_t launch_shard_copy(const DevState &d, bool exp, uint32_t r0, uint32_t
 }
 
 // ---------------------------------------------------------------------------
-// dm_hash_prompts: full cache keys of every block, plus the two positions.
-__global__ void k_hash_keys(DevState d, uint32_t n, uint64_t *keys, uint64_t *key_off, uint64_t *pos) {
+// dm_hash_prompts and its allocation-free variant, after the hashing kernel:
+// the cache keys of every block from the local prefix values (which may lie
+// in the key buffer itself), the key offsets and the two ring positions.
+// A CTA takes 32 consecutive segments: all its threads sum the totals of the
+// earlier segments of the first one's request, one warp scans the 32 totals
+// from there (restarting where a request starts), then each warp turns four
+// segments' prefix values into keys.
+// Bound: the prefix values' read and the keys' write.  With a warp per
+// request, walking it 32 blocks per round trip, 512 prompts of 32k-131k
+// tokens took 134 us in 64 CTAs (GB300), now 14.7; the whole call went from
+// 122 to 51 us.
+constexpr uint32_t kKeySegs = 32;
+__global__ void __launch_bounds__(256) k_hash_keys(DevState d, uint32_t n, uint64_t *keys, uint64_t *key_off,
+                                                   uint64_t *pos) {
+    pdl_enter();
     if (has_err(d.err)) return;
-    const int lane = threadIdx.x & 31;
-    const uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (r >= n) return;
-    request_carries(d, r, lane);
-    __syncwarp();
-    const uint32_t nblk = d.r_nblk[r], s0 = d.r_segoff[r];
-    const uint64_t bo = d.r_blkoff[r];
-    for (uint32_t b = lane; b < nblk; b += 32)
-        keys[bo + b] = cache_key(d.plocal[bo + b] + d.seg_carry[s0 + b / kSegBlocks], d.Sc);
-    uint64_t p1, p2;
-    route_positions(d, r, lane, p1, p2);
-    if (lane == 0) {
-        key_off[r] = bo;
-        pos[2 * r] = p1;
-        pos[2 * r + 1] = p2;
-        if (r == n - 1) key_off[n] = bo + nblk;
+    __shared__ uint64_t s_carry[kKeySegs], s_sum[8];
+    __shared__ uint32_t s_req[kKeySegs], s_j[kKeySegs];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t total = d.info->total_segs;
+    for (uint64_t c0 = uint64_t(blockIdx.x) * kKeySegs; c0 < total; c0 += uint64_t(gridDim.x) * kKeySegs) {
+        const uint32_t seg0 = (uint32_t)c0, m = min(kKeySegs, total - seg0);
+        const uint32_t first = d.r_segoff[d.seg_req[seg0]];
+        uint64_t v = 0;
+        for (uint32_t x = first + threadIdx.x; x < seg0; x += blockDim.x) v += d.seg_total[x];
+        v = warp_sum_u64(v);
+        if (lane == 0) s_sum[wid] = v;
+        __syncthreads();
+        if (wid == 0) {
+            uint64_t in = lane < 8 ? s_sum[lane] : 0;
+            in = warp_sum_u64(in);
+            const bool valid = (uint32_t)lane < m;
+            const uint32_t r = valid ? d.seg_req[seg0 + lane] : 0;
+            const uint32_t j = valid ? seg0 + lane - d.r_segoff[r] : 0;
+            const uint64_t t = valid ? d.seg_total[seg0 + lane] : 0;
+            const uint64_t ex = warp_incl_scan(t, lane) - t;
+            // its request's first segment in this chunk: lane - j, or before the chunk
+            const uint64_t at = shfl_u64(ex, j <= (uint32_t)lane ? lane - j : 0);
+            if (valid) {
+                s_carry[lane] = j <= (uint32_t)lane ? ex - at : in + ex;
+                s_req[lane] = r;
+                s_j[lane] = j;
+            }
+        }
+        __syncthreads();
+        uint64_t P[4][2];
+        uint32_t nblk[4];
+        uint64_t bo[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t x = wid * 4 + q;
+            nblk[q] = 0;
+            if (x < m) {
+                const uint32_t r = s_req[x], b0 = s_j[x] * kSegBlocks;
+                nblk[q] = d.r_nblk[r];
+                bo[q] = d.r_blkoff[r];
+                const uint64_t *pl = d.plocal + bo[q] + b0;
+                P[q][0] = b0 + lane < nblk[q] ? pl[lane] : 0;
+                P[q][1] = b0 + lane + 32 < nblk[q] ? pl[lane + 32] : 0;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t x = wid * 4 + q;
+            if (x >= m) continue;
+            const uint32_t r = s_req[x], j = s_j[x], b0 = j * kSegBlocks;
+            const uint64_t carry = s_carry[x];
+            uint64_t *out = keys + bo[q] + b0;
+            if (b0 + lane < nblk[q]) out[lane] = cache_key(P[q][0] + carry, d.Sc);
+            if (b0 + lane + 32 < nblk[q]) out[lane + 32] = cache_key(P[q][1] + carry, d.Sc);
+            const uint32_t kk = min(d.Kroute, nblk[q]) - 1 - b0;   // block K-1 in this segment, if any
+            if (kk < kSegBlocks) {
+                const uint64_t P1 = shfl_u64(kk < 32 ? P[q][0] : P[q][1], kk & 31) + carry;
+                // f2 ran over blocks < K only: segments 0 .. j (at most 4)
+                const uint64_t p2 = warp_sum_u64((uint32_t)lane <= j ? d.seg_total2[seg0 + x - j + lane] : 0);
+                if (lane == 0) {
+                    pos[2 * r] = fmix64(P1 ^ d.Sr1);
+                    pos[2 * r + 1] = fmix64(p2 ^ d.Sr2);
+                }
+            }
+            if (j == 0 && lane == 0) {
+                key_off[r] = bo[q];
+                if (r == n - 1) key_off[n] = bo[q] + nblk[q];
+            }
+        }
+        __syncthreads();   // the chunk's values are read before the next one's are written
     }
 }
 
-cudaError_t launch_hash_keys(const DevState &d, uint32_t n, uint64_t *keys, uint64_t *key_off,
-                             uint64_t *pos, cudaStream_t st) {
-    if (n == 0) return cudaSuccess;
-    const uint32_t warps = 8;
-    k_hash_keys<<<(n + warps - 1) / warps, warps * 32, 0, st>>>(d, n, keys, key_off, pos);
+cudaError_t launch_hash_keys(const DevState &d, const dm_batch &b, uint64_t *keys, uint64_t *key_off, uint64_t *pos,
+                             cudaStream_t st) {
+    if (b.n == 0) return cudaSuccess;
+    // segments of the batch, at most
+    const uint64_t segs = b.total_tokens / d.B / kSegBlocks + b.n;
+    const unsigned grid = (unsigned)std::min<uint64_t>((segs + kKeySegs - 1) / kKeySegs, 1u << 20);
+    DM_TRY(launch_pdl(k_hash_keys, grid, 256, 0, st, d, b.n, keys, key_off, pos));
     return cudaGetLastError();
 }
 

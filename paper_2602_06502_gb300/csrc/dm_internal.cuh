@@ -524,24 +524,6 @@ __device__ __forceinline__ void carries_role(const DevState &d, const dm_route_o
     }
 }
 
-// The two ring positions of request r (after request_carries): P^1_{K-1}
-// from its local prefix value plus carry, P^2_{K-1} as the sum of the f2
-// segment partials (f2 only runs over blocks < K).  Whole warp; all lanes
-// return the same values.
-__device__ __forceinline__ void route_positions(const DevState &d, uint32_t r, int lane, uint64_t &pos1,
-                                                uint64_t &pos2) {
-    const uint32_t nblk = d.r_nblk[r], s0 = d.r_segoff[r];
-    const uint32_t K = min(d.Kroute, nblk);
-    const uint32_t last = (K - 1) / kSegBlocks;   // segments holding blocks < K: 0..last
-    const uint64_t P1 = d.plocal[d.r_blkoff[r] + K - 1] + d.seg_carry[s0 + last];
-    uint64_t p2 = 0;
-    for (uint32_t j = lane; j <= last; j += 32) p2 += d.seg_total2[s0 + j];
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) p2 += shfl_xor_u64(p2, o);
-    pos1 = fmix64(P1 ^ d.Sr1);
-    pos2 = fmix64(p2 ^ d.Sr2);
-}
-
 // ---------------------------------------------------------------------------
 // Adaptive prefix tree tables (open addressing, linear probing, bounded).
 
@@ -685,27 +667,6 @@ __device__ __forceinline__ void drain_queue(const DevState &d, uint32_t i, uint6
     }
 }
 
-// The same two ring positions without the stored carries: the carry of the
-// segment holding block K-1 is summed here from the (at most 4) segment
-// totals before it, so the ring search need not wait for request_carries.
-// Whole warp; all lanes return the same values.
-__device__ __forceinline__ void route_positions_direct(const DevState &d, uint32_t r, int lane, uint64_t &pos1,
-                                                       uint64_t &pos2) {
-    const uint32_t nblk = d.r_nblk[r], s0 = d.r_segoff[r];
-    const uint32_t K = min(d.Kroute, nblk);
-    const uint32_t last = (K - 1) / kSegBlocks;   // <= 3 (K <= 256)
-    uint64_t c = (uint32_t)lane < last ? d.seg_total[s0 + lane] : 0;
-    uint64_t p2 = (uint32_t)lane <= last ? d.seg_total2[s0 + lane] : 0;
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-        c += shfl_xor_u64(c, o);
-        p2 += shfl_xor_u64(p2, o);
-    }
-    const uint64_t P1 = d.plocal[d.r_blkoff[r] + K - 1] + c;
-    pos1 = fmix64(P1 ^ d.Sr1);
-    pos2 = fmix64(p2 ^ d.Sr2);
-}
-
 // ---------------------------------------------------------------------------
 // Routing helpers (Sec. 3.2, Sec. 3.4, App. A.1.3, App. A.3.2).
 
@@ -834,8 +795,8 @@ cudaError_t launch_choice(const DevState &d, const dm_route_out &o, uint32_t n, 
 cudaError_t launch_commit(const DevState &d, uint32_t n, cudaStream_t st);
 cudaError_t launch_rebalance(const DevState &d, uint32_t n, uint64_t seq0, uint32_t call,
                              dm_migration *out, uint32_t cap, uint32_t *n_out, cudaStream_t st);
-cudaError_t launch_hash_keys(const DevState &d, uint32_t n, uint64_t *keys, uint64_t *key_off,
-                             uint64_t *pos, cudaStream_t st);
+cudaError_t launch_hash_keys(const DevState &d, const dm_batch &b, uint64_t *keys, uint64_t *key_off, uint64_t *pos,
+                             cudaStream_t st);
 cudaError_t launch_ring_lookup(const DevState &d, const uint64_t *pos, uint32_t n, uint32_t *o1,
                                uint32_t *o2, cudaStream_t st);
 cudaError_t launch_ring_update(DevState &d, uint32_t id, bool add, uint64_t *scratch_pos, uint32_t *scratch_vidx,

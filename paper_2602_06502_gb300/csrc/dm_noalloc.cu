@@ -25,8 +25,7 @@ constexpr size_t kOffBlkoff = kOffTokoff + align256(8 * kNaReq);
 constexpr size_t kOffSegReq = kOffBlkoff + align256(8 * kNaReq);
 constexpr size_t kOffSegTot = kOffSegReq + align256(4 * kNaSegs);
 constexpr size_t kOffSegTot2 = kOffSegTot + align256(8 * kNaSegs);
-constexpr size_t kOffSegCarry = kOffSegTot2 + align256(8 * kNaSegs);
-constexpr size_t kOffInfo = kOffSegCarry + align256(8 * kNaSegs);
+constexpr size_t kOffInfo = kOffSegTot2 + align256(8 * kNaSegs);
 constexpr size_t kOffErr = kOffInfo + align256(sizeof(BatchInfo));
 constexpr size_t kScratchBytes = kOffErr + 256;
 
@@ -60,30 +59,6 @@ uint64_t na_splitmix_next(uint64_t &s) {
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
     return z ^ (z >> 31);
-}
-
-// Warp per request: ring positions from the prefix values, then the prefix
-// values in the caller's buffer become cache keys in place.
-__global__ void k_na_finish(DevState d, uint32_t n, uint64_t *keys, uint64_t *key_off, uint64_t *pos) {
-    if (has_err(d.err)) return;
-    const int lane = threadIdx.x & 31;
-    const uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (r >= n) return;
-    request_carries(d, r, lane);
-    __syncwarp();
-    uint64_t p1, p2;
-    route_positions(d, r, lane, p1, p2);   // reads the prefix value of block K-1
-    __syncwarp();
-    const uint32_t nblk = d.r_nblk[r], s0 = d.r_segoff[r];
-    const uint64_t bo = d.r_blkoff[r];
-    for (uint32_t b = lane; b < nblk; b += 32)
-        keys[bo + b] = cache_key(keys[bo + b] + d.seg_carry[s0 + b / kSegBlocks], d.Sc);
-    if (lane == 0) {
-        key_off[r] = bo;
-        pos[2 * r] = p1;
-        pos[2 * r + 1] = p2;
-        if (r == n - 1) key_off[n] = bo + nblk;
-    }
 }
 
 }  // namespace
@@ -134,7 +109,6 @@ extern "C" DM_API dm_status dm_hash_prompts_noalloc(uint32_t block_tokens, uint3
     d.seg_req = reinterpret_cast<uint32_t *>(base + kOffSegReq);
     d.seg_total = reinterpret_cast<uint64_t *>(base + kOffSegTot);
     d.seg_total2 = reinterpret_cast<uint64_t *>(base + kOffSegTot2);
-    d.seg_carry = reinterpret_cast<uint64_t *>(base + kOffSegCarry);
     d.info = reinterpret_cast<BatchInfo *>(base + kOffInfo);
     d.err = reinterpret_cast<uint32_t *>(base + kOffErr);
     d.plocal = keys_dev;   // prefix values live in the output until converted
@@ -144,10 +118,7 @@ extern "C" DM_API dm_status dm_hash_prompts_noalloc(uint32_t block_tokens, uint3
     e = cudaMemsetAsync(d.err, 0, sizeof(uint32_t), st);
     if (e == cudaSuccess) e = launch_setup(d, *b, st);
     if (e == cudaSuccess) e = launch_hash(d, *b, hash_grid_size(), st);
-    if (e == cudaSuccess) {
-        k_na_finish<<<(b->n + 7) / 8, 256, 0, st>>>(d, b->n, keys_dev, key_off_dev, pos_dev);
-        e = cudaGetLastError();
-    }
+    if (e == cudaSuccess) e = launch_hash_keys(d, *b, keys_dev, key_off_dev, pos_dev, st);   // in place
     uint32_t err = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&err, d.err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);

@@ -1,7 +1,7 @@
 // dm_setup.cu -- batch set-up: validation of the prompts, per-request block
 // and segment offsets (and, for routing, the offsets of the hashing order),
-// the segment -> request map of the hashing-only calls, and (in the same
-// launch as the set-up, routing calls only) the queue drain of Sec. 3.2.
+// and (in the same launch as the set-up, routing calls only) the queue drain
+// of Sec. 3.2.
 #include "dm_internal.cuh"
 
 namespace dm {
@@ -113,38 +113,24 @@ __global__ void __launch_bounds__(1024) k_setup(DevState d, const uint64_t *off,
     }
 }
 
-// Segment -> request map, one warp per request.
-__global__ void k_segmap(DevState d, uint32_t n) {
-    pdl_enter();
-    if (has_err(d.err)) return;
-    const int lane = threadIdx.x & 31;
-    const uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (r >= n) return;
-    const uint32_t s0 = d.r_segoff[r];
-    const uint32_t ns = (d.r_nblk[r] + kSegBlocks - 1) / kSegBlocks;
-    for (uint32_t j = lane; j < ns; j += 32) d.seg_req[s0 + j] = r;
-}
-
 cudaError_t launch_setup(const DevState &d, const dm_batch &b, cudaStream_t st) {
     DM_TRY(launch_pdl(k_setup<false>, 1, 1024, 0, st, d, b.offsets, b.lengths, b.n, b.total_tokens, uint64_t(0),
                       uint64_t(0)));
-    if (b.n) DM_TRY(launch_pdl(k_segmap, (b.n + 7) / 8, 256, 0, st, d, b.n));
     return cudaGetLastError();
 }
 
-// Routing with d candidates: the plain layout (segment order, then the
-// segment -> request map), the CV fold and the queue drain.
+// Routing with d candidates: the plain layout (segment order), the CV fold
+// and the queue drain.
 cudaError_t launch_setup_plain_drain(const DevState &d, const dm_batch &b, uint64_t delta, uint64_t t0,
                                      cudaStream_t st) {
     const unsigned drain_ctas = (d.M + 31) / 32;
     DM_TRY(launch_pdl(k_setup<false>, 2 + drain_ctas, 1024, 0, st, d, b.offsets, b.lengths, b.n, b.total_tokens,
                       delta, t0));
-    if (b.n) DM_TRY(launch_pdl(k_segmap, (b.n + 7) / 8, 256, 0, st, d, b.n));
     return cudaGetLastError();
 }
 
-// Routing: the layout in the hashing order of k_hash_probe (which writes
-// the segment -> request map itself), the CV fold and the queue drain.
+// Routing: the layout in the hashing order of k_hash_probe, the CV fold and
+// the queue drain.
 cudaError_t launch_setup_route(const DevState &d, const dm_batch &b, uint64_t delta, uint64_t t0,
                                cudaStream_t st) {
     const unsigned drain_ctas = (d.M + 31) / 32;
