@@ -342,8 +342,8 @@ dm_status dm_create(const dm_config *cfg, dm_handle **out) {
     A(dalloc(h, &d.inst_state, M));
     A(dalloc(h, &d.next_live, M));
     A(dalloc(h, &d.W, M));
-    A(dalloc(h, &d.q_head, M));
-    A(dalloc(h, &d.q_tail, M));
+    A(dalloc(h, &d.q_head, 2 * M));   // heads, then tails (one copy reads both of an id)
+    d.q_tail = d.q_head + M;
     A(dalloc(h, &d.q, M * d.Q));
     A(dalloc(h, &d.table, M));
     A(dalloc(h, &d.logbuf, M));
@@ -517,29 +517,20 @@ static void sync_copy(dm_handle *h) {
 
 static dm_status ring_change(dm_handle *h, uint32_t id, bool add) {
     DevState &d = h->d;
-    const uint32_t newR = add ? d.R + d.V : d.R - d.V;
-    uint64_t *nv[dm::kMaxD] = {};
-    uint32_t *no[dm::kMaxD] = {}, *ni[dm::kMaxD] = {};
+    DevState next = d;
     for (uint32_t f = 0; f < d.nrings; ++f) {
         const int nb = 1 - h->cur[f];
-        nv[f] = h->vpos_buf[f][nb];
-        no[f] = h->owner_buf[f][nb];
-        ni[f] = h->vidx_buf[f][nb];
+        next.ring[f].vpos = h->vpos_buf[f][nb];
+        next.ring[f].owner = h->owner_buf[f][nb];
+        next.ring[f].vidx = h->vidx_buf[f][nb];
     }
-    cudaError_t e = dm::launch_ring_update(d, id, add, h->ring_spos, h->ring_svidx, nv, no, ni, h->st);
+    set_levels(next, add ? d.R + d.V : d.R - d.V);
+    const cudaError_t e = dm::launch_ring_update(d, next, id, add, h->ring_spos, h->ring_svidx, h->st);
     if (e != cudaSuccess) return map_cuda(h, e);
-    for (uint32_t f = 0; f < d.nrings; ++f) {
-        h->cur[f] = 1 - h->cur[f];
-        d.ring[f].vpos = nv[f];
-        d.ring[f].owner = no[f];
-        d.ring[f].vidx = ni[f];
-    }
-    set_levels(d, newR);
-    e = dm::launch_tree_build(d, h->st);
-    if (e == cudaSuccess) e = dm::launch_set_state(d, id, add ? 1 : 2, h->st);
-    if (e == cudaSuccess) e = dm::launch_next_live(d, h->st);
+    for (uint32_t f = 0; f < d.nrings; ++f) h->cur[f] = 1 - h->cur[f];
+    d = next;
     sync_copy(h);
-    return map_cuda(h, e);
+    return DM_OK;
 }
 
 dm_status dm_add_instance(dm_handle *h, uint32_t id) {
@@ -551,16 +542,14 @@ dm_status dm_add_instance(dm_handle *h, uint32_t id) {
     if (h->state[id] == 1) return DM_ERR_DUPLICATE_ID;
     cudaError_t e = cudaSuccess;
     if (h->state[id] == 2) {
-        uint32_t ht[2];
-        e = cudaMemcpyAsync(&ht[0], d.q_head + id, 4, cudaMemcpyDeviceToHost, h->st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&ht[1], d.q_tail + id, 4, cudaMemcpyDeviceToHost, h->st);
+        uint32_t ht[2];   // its queue's head and tail (q_tail follows q_head, M entries on)
+        e = cudaMemcpy2DAsync(ht, 4, d.q_head + id, 4ull * d.M, 4, 2, cudaMemcpyDeviceToHost, h->st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
         if (e != cudaSuccess) return map_cuda(h, e);
         if (ht[0] != ht[1]) return DM_ERR_DUPLICATE_ID;
     }
-    Slot *cur = h->tables[id];   // the index this id uses now (rebuilds trade buffers with the pool)
-    const bool first = cur == nullptr;
-    if (first) {
+    dm::InstanceBuffers ib{};
+    if (!h->tables[id]) {   // never added before (a re-added id keeps whichever index buffer it holds now)
         Slot *t = nullptr, *spare = nullptr;
         Rec *lg = nullptr, *lg2 = nullptr;
         uint8_t *sf = nullptr, *sf2 = nullptr;
@@ -574,14 +563,9 @@ dm_status dm_add_instance(dm_handle *h, uint32_t id) {
         if (e == cudaSuccess) e = dalloc(h, &hm, d.logcap);
         if (e == cudaSuccess) e = dalloc(h, &hm2, d.logcap);
         if (e != cudaSuccess) { cudaGetLastError(); return DM_ERR_OOM; }
-        if (spare) {
-            e = cudaMemcpyAsync(d.pool + d.pool_n, &spare, sizeof(Slot *), cudaMemcpyHostToDevice, h->st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
-            if (e != cudaSuccess) return map_cuda(h, e);
-            ++h->d.pool_n;
-        }
         h->tables[id] = t;
-        cur = t;
+        ib.table = t;
+        ib.spare = spare;
         h->logs[id] = lg;
         h->logs2[id] = lg2;
         h->stales[id] = sf;
@@ -589,32 +573,15 @@ dm_status dm_add_instance(dm_handle *h, uint32_t id) {
         h->homes[id] = hm;
         h->homes2[id] = hm2;
     }
-    if (!first) {   // a re-added id keeps whichever index buffer it holds now
-        e = cudaMemcpyAsync(&cur, d.table + id, sizeof(Slot *), cudaMemcpyDeviceToHost, h->st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
-        if (e != cudaSuccess) return map_cuda(h, e);
-    }
-    // a (re-)added instance starts empty, both buffers of each log
-    struct { void *dst; const void *src; } ptrs[] = {
-        {d.table + id, &cur},
-        {d.logbuf + id, &h->logs[id]}, {d.logbuf_alt + id, &h->logs2[id]},
-        {d.stale + id, &h->stales[id]}, {d.stale_alt + id, &h->stales2[id]},
-        {d.loghome + id, &h->homes[id]}, {d.loghome_alt + id, &h->homes2[id]}};
-    for (auto &pp : ptrs)
-        if (e == cudaSuccess) e = cudaMemcpyAsync(pp.dst, pp.src, sizeof(void *), cudaMemcpyHostToDevice, h->st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
+    ib.log[0] = h->logs[id];
+    ib.log[1] = h->logs2[id];
+    ib.stale[0] = h->stales[id];
+    ib.stale[1] = h->stales2[id];
+    ib.home[0] = h->homes[id];
+    ib.home[1] = h->homes2[id];
+    e = dm::launch_reset_instance(d, id, ib, h->st);
     if (e != cudaSuccess) return map_cuda(h, e);
-    e = cudaMemsetAsync(cur, 0, d.S * sizeof(Slot), h->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->stales[id], 0, d.logcap, h->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->stales2[id], 0, d.logcap, h->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.log_front + id, 0, 8, h->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.log_tail + id, 0, 8, h->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.live + id, 0, 8, h->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.used + id, 0, 8, h->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.W + id, 0, 8, h->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.q_head + id, 0, 4, h->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.q_tail + id, 0, 4, h->st);
-    if (e != cudaSuccess) return map_cuda(h, e);
+    if (ib.spare) ++d.pool_n;
     s = ring_change(h, id, true);
     if (s) return s;
     h->state[id] = 1;

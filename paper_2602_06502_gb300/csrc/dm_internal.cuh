@@ -311,10 +311,10 @@ __device__ __forceinline__ void pdl_enter() {
 // Launch a kernel that begins with pdl_enter() with programmatic stream
 // serialization.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t st,
                               Args... args) {
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -799,11 +799,18 @@ cudaError_t launch_hash_keys(const DevState &d, const dm_batch &b, uint64_t *key
                              cudaStream_t st);
 cudaError_t launch_ring_lookup(const DevState &d, const uint64_t *pos, uint32_t n, uint32_t *o1,
                                uint32_t *o2, cudaStream_t st);
-cudaError_t launch_ring_update(DevState &d, uint32_t id, bool add, uint64_t *scratch_pos, uint32_t *scratch_vidx,
-                               uint64_t *const *new_vpos, uint32_t *const *new_owner, uint32_t *const *new_vidx,
-                               cudaStream_t st);
-cudaError_t launch_tree_build(const DevState &d, cudaStream_t st);
+// next: the ring buffers and levels after the update
+cudaError_t launch_ring_update(DevState &d, const DevState &next, uint32_t id, bool add, uint64_t *scratch_pos,
+                               uint32_t *scratch_vidx, cudaStream_t st);
 cudaError_t launch_next_live(const DevState &d, cudaStream_t st);
-cudaError_t launch_set_state(const DevState &d, uint32_t id, uint8_t s, cudaStream_t st);
+// Buffers of one instance: its index (null: keep the one it has) and a spare
+// one for the pool (or null), and both buffers of each of its logs.
+struct InstanceBuffers {
+    Slot *table, *spare;
+    Rec *log[2];
+    uint8_t *stale[2];
+    uint32_t *home[2];
+};
+cudaError_t launch_reset_instance(const DevState &d, uint32_t id, const InstanceBuffers &b, cudaStream_t st);
 
 }  // namespace dm
