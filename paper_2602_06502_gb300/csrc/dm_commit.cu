@@ -25,7 +25,7 @@ namespace cg = cooperative_groups;
 namespace dm {
 
 constexpr int kMtThreads = 256;
-constexpr uint32_t kPrepChunk = 1024;
+constexpr uint32_t kPrepVec = 4;        // requests per thread whose loads the commit prep issues together
 constexpr uint32_t kFlagCompact = 1, kFlagRebuild = 2;
 constexpr uint32_t kZeroChunk = 4096;   // slots or flag bytes cleared per chunk
 
@@ -208,26 +208,12 @@ static size_t plan_smem(uint32_t M) { return size_t(M) * 24 + 8; }
 // The plan, computed by a whole CTA; `store`: also write it to global
 // memory (flags, chunk offsets, pool slots and buffers, the rotation start
 // the commit prep installs, the counters of this commit).
-__device__ void maint_plan_cta(const DevState &d, uint32_t n, const PlanSm &P, bool store) {
+__device__ void maint_plan_cta(const DevState &d, const PlanSm &P, bool store) {
     __shared__ uint32_t s_w[33];
     __shared__ uint32_t s_served, s_last;
-    // blocks each instance receives: the choice kernel's count, unless a
-    // rebalance has moved a request of the batch since
-    const bool dirty = d.info->final_dirty != 0;
-    for (uint32_t i = threadIdx.x; i < d.M; i += blockDim.x) P.cnt[i] = dirty ? 0 : d.log_adv[i];
-    __syncthreads();
-    for (uint32_t r0 = threadIdx.x; dirty && r0 < n; r0 += 4 * blockDim.x) {   // four loads in flight per thread
-        uint32_t f[4], nb[4];
-#pragma unroll
-        for (uint32_t u = 0; u < 4; ++u) {
-            const uint32_t r = r0 + u * blockDim.x;
-            f[u] = r < n ? d.r_final[r] : 0;
-            nb[u] = r < n ? d.r_nblk[r] : 0;
-        }
-#pragma unroll
-        for (uint32_t u = 0; u < 4; ++u)
-            if (nb[u]) atomicAdd(reinterpret_cast<unsigned long long *>(&P.cnt[f[u]]), (unsigned long long)nb[u]);
-    }
+    // blocks each instance receives: the choice kernel's counts, kept current
+    // by a rebalance that moves requests of the batch
+    for (uint32_t i = threadIdx.x; i < d.M; i += blockDim.x) P.cnt[i] = d.log_adv[i];
     __syncthreads();
     // 1) what each instance needs: compaction if its log would overflow,
     //    a rebuild if its index would pass rb_thr taken slots
@@ -348,14 +334,14 @@ __device__ void compact_scan_cta(const DevState &d, const PlanSm &P) {
     }
 }
 
-// n: requests of the batch; dynamic smem: plan_smem(M) bytes.
-__global__ void __launch_bounds__(kMtThreads) k_maint_a(DevState d, uint32_t n) {
+// Dynamic smem: plan_smem(M) bytes.
+__global__ void __launch_bounds__(kMtThreads) k_maint_a(DevState d) {
     pdl_enter();
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint32_t s_i, s_cnt[kMtThreads / 32];
     if (has_err(d.err)) return;
     const PlanSm P = plan_sm(smem, d.M);
-    maint_plan_cta(d, n, P, blockIdx.x == 0);
+    maint_plan_cta(d, P, blockIdx.x == 0);
     // clearing: a rebuilding instance's chunks cover its second index first,
     // a compacting instance's (then) its second stale-flag array
     const uint32_t nz = P.mr[d.M];
@@ -468,11 +454,10 @@ __global__ void __launch_bounds__(kMtThreads) k_maint_c(DevState d, uint32_t n) 
 // this commit and advance its tail.  The choice kernel already placed every
 // request among its instance's records; only when a rebalance moved a
 // request of this batch are the offsets recomputed (arrival order per final
-// instance).  One CTA, after every CTA of k_maint_c; adv: one u64 per
+// instance), a warp per 32 requests: one thread walking 4,096 requests took
+// 200 us of a rebalanced pass (256 instances, GB300).  One CTA, after every CTA of k_maint_c; adv: one u64 per
 // instance in shared memory.
 __device__ void commit_prep_cta(const DevState &d, uint32_t n, uint64_t *adv) {
-    __shared__ uint32_t s_f[kPrepChunk], s_nb[kPrepChunk];
-    __shared__ uint64_t s_off[kPrepChunk];
     for (uint32_t i = threadIdx.x; i < d.M; i += blockDim.x) {
         const uint32_t fl = d.mt_flags[i];
         if (fl & kFlagCompact) {
@@ -501,23 +486,24 @@ __device__ void commit_prep_cta(const DevState &d, uint32_t n, uint64_t *adv) {
     if (dirty) {
         __syncthreads();
         for (uint32_t i = threadIdx.x; i < d.M; i += blockDim.x) adv[i] = 0;
-        for (uint32_t base = 0; base < n; base += kPrepChunk) {
-            const uint32_t m = min(kPrepChunk, n - base);
-            __syncthreads();
-            for (uint32_t k = threadIdx.x; k < m; k += blockDim.x) {
-                s_f[k] = d.r_final[base + k];
-                s_nb[k] = d.r_nblk[base + k];
+        __syncthreads();
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        for (uint32_t base = 0; base < n; base += kPrepVec * kMtThreads) {
+            uint32_t f[kPrepVec], nb[kPrepVec];
+#pragma unroll
+            for (uint32_t u = 0; u < kPrepVec; ++u) {
+                const uint32_t r = base + u * kMtThreads + threadIdx.x;
+                f[u] = r < n ? d.r_final[r] : 0;
+                nb[u] = r < n ? d.r_nblk[r] : 0;
             }
-            __syncthreads();
-            if (threadIdx.x == 0)
-                for (uint32_t k = 0; k < m; ++k) {
-                    const uint32_t f = s_f[k];
-                    const uint64_t o = adv[f];
-                    s_off[k] = o;
-                    adv[f] = o + s_nb[k];
-                }
-            __syncthreads();
-            for (uint32_t k = threadIdx.x; k < m; k += blockDim.x) d.r_touchoff[base + k] = s_off[k];
+#pragma unroll
+            for (uint32_t u = 0; u < kPrepVec; ++u) {
+                const uint32_t b0 = base + u * kMtThreads;
+                if (b0 >= n) break;
+                const uint32_t r = b0 + threadIdx.x, m = min(uint32_t(kMtThreads), n - b0);
+                const uint64_t off = record_place<kMtThreads>(adv, f[u], nb[u], r < n, wid, (m + 31) / 32, lane);
+                if (r < n) d.r_touchoff[r] = off;
+            }
         }
         __syncthreads();
     }
@@ -962,12 +948,12 @@ cudaError_t launch_commit(const DevState &d, uint32_t n, cudaStream_t st) {
         if (e != cudaSuccess) return e;
         configured = smem_a;
     }
-    // every CTA of k_maint_a reads the whole batch for its plan: two per SM
+    // every CTA of k_maint_a computes the plan over all instances: two per SM
     static const int g_a = full_grid(k_maint_a, kMtThreads) < 2 * sm_count() ? full_grid(k_maint_a, kMtThreads)
                                                                                 : 2 * sm_count(),
                      g_c = full_grid(k_maint_c, kMtThreads), g_t = full_grid(k_commit_touch, kTouchThreads),
                      g_ev = evict_grid();
-    DM_TRY(launch_pdl(k_maint_a, g_a, kMtThreads, smem_a, st, d, n));
+    DM_TRY(launch_pdl(k_maint_a, g_a, kMtThreads, smem_a, st, d));
     DM_TRY(launch_pdl(k_maint_c, g_c, kMtThreads, smem_c, st, d, n));
     DM_TRY(launch_pdl(k_commit_touch, g_t, kTouchThreads, 0, st, d));
     DM_TRY(launch_pdl(k_evict, g_ev, kEvThreads, 0, st, d));

@@ -668,6 +668,44 @@ __device__ __forceinline__ void drain_queue(const DevState &d, uint32_t i, uint6
 }
 
 // ---------------------------------------------------------------------------
+// Running sums per instance over a chunk of requests in arrival order: returns
+// PT[ch] as the request finds it and moves it on by `step` (the choice counts
+// records of this batch << 32 | queue tail, so its step is (the request's
+// blocks << 32) + 1).  Called by the kChunk threads of one chunk, a warp per
+// window of 32 requests, in window order over a barrier of their own (valid:
+// the lane has a request; PT in shared memory).
+template <uint32_t kChunk>
+__device__ __forceinline__ uint64_t record_place(uint64_t *PT, uint32_t ch, uint64_t step, bool valid,
+                                                 uint32_t window, uint32_t windows, int lane) {
+    const uint32_t peers = __match_any_sync(0xffffffffu, valid ? ch : 0x80000000u | lane);
+    const uint32_t lower = peers & ((1u << lane) - 1u);
+    // inclusive sum over the peers up to this lane, by pointer jumping
+    int prev = lower ? 31 - __clz(lower) : -1;
+    uint64_t sum = step;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const uint64_t u = shfl_u64(sum, prev & 31);
+        const int pp = __shfl_sync(0xffffffffu, prev, prev & 31);
+        if (prev >= 0) {
+            sum += u;
+            prev = pp;
+        }
+    }
+    const bool last = (peers >> lane) == 1u;
+    uint64_t place = 0;
+    for (uint32_t w = 0; w < windows; ++w) {
+        if (w == window) {
+            const uint64_t p = valid ? PT[ch] : 0;
+            place = p + sum - step;
+            __syncwarp();
+            if (valid && last) PT[ch] = p + sum;
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(kChunk) : "memory");
+    }
+    return place;
+}
+
+// ---------------------------------------------------------------------------
 // Routing helpers (Sec. 3.2, Sec. 3.4, App. A.1.3, App. A.3.2).
 
 __device__ __forceinline__ const uint64_t *level_ptr(const DevState &d, int f, int k) {

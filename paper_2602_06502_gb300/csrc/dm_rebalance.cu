@@ -404,6 +404,9 @@ __global__ void __launch_bounds__(1024) k_rebalance(DevState d, uint32_t n, uint
                 if (e.seq >= seq0 && e.seq < seq0 + n) {
                     d.r_final[e.seq - seq0] = j;
                     d.info->final_dirty = 1;
+                    const uint64_t nb = e.L / d.B;   // its log records move too
+                    atomicAdd(reinterpret_cast<unsigned long long *>(d.log_adv + i), (unsigned long long)-nb);
+                    atomicAdd(reinterpret_cast<unsigned long long *>(d.log_adv + j), (unsigned long long)nb);
                     if (fresh) d.r_koff[e.seq - seq0] = e.koff;   // the commit writes its keys there
                 }
                 if (cnt0 + t < cap) out[cnt0 + t] = dm_migration{e.seq, i, j};
