@@ -20,6 +20,7 @@
 //
 // At the end of the file: routing with d candidates (App. A.8).
 #include <algorithm>
+#include <type_traits>
 
 #include "dm_internal.cuh"
 
@@ -428,27 +429,33 @@ __global__ void __launch_bounds__(kAllBlock) k_probe_all(DevState d, uint32_t n)
 // ---------------------------------------------------------------------------
 // The cluster-wide choice over up to 512 instances, pipelined like the pair
 // choice.  Every request depends on the one before it, so the chain is the
-// argmin over the instances: their loads stay in the deciding warp's
-// registers (lane l holds the live ids of list indices J l .. J l + J - 1),
-// as 32-bit offsets from the smallest load, and one request is J compares, a
-// 32-bit minimum over the warp, a vote, and an add in the winning lane.  The
-// lowest lane with the smallest key holds the lowest id.  A chunk whose
-// loads and work do not fit 31 bits is decided in 64 bits instead.  The hits
-// come into shared memory a chunk ahead.
+// argmin over the instances and it alone is left to the deciding warp: the
+// loads stay in its registers (lane l holds the live ids of list indices
+// J l .. J l + J - 1), as 32-bit offsets from the smallest load, and one
+// request is J compares, a 32-bit minimum over the warp, a vote, and an add in
+// the winning lane, which stores the index it holds.  The lowest lane with the
+// smallest key holds the lowest id.  A chunk whose loads and work do not fit
+// 31 bits is decided in 64 bits instead.  The hits come into shared memory a
+// chunk ahead; the loads that a request found on its candidates follow from
+// the loads at the chunk's start and the choices before it, which the emitting
+// warps add up.
 // 4,096 agent prompts on 64 instances, min TTFT, GB300: 1,678 us with 64-bit
 // keys and loads in shared memory, three reductions a request, and staging
-// and emission between the chunks; 922 us so.
+// and emission between the chunks; 922 us when the deciding warp also read
+// and wrote the loads in shared memory for every request, 1,247 us a pass;
+// 680 us a pass so.
 constexpr uint32_t kGlobalStageThreads = 256;
 template <uint32_t J>
 struct GlobalPipe {
     static constexpr uint32_t kChunk = J <= 8 ? 64 : 32;   // three buffers of hits fit at 512 instances
     static constexpr uint32_t kThreads = Pipe<kChunk, kGlobalStageThreads>::kThreads;
     struct Stage {
-        uint32_t hit[kChunk][32 * J];
-        uint64_t cl[kChunk];                    // cost x L
-        uint64_t t[2][kChunk], wch[kChunk];     // loads of c1 and c2 before, of the choice after
-        uint32_t ci[2][kChunk], hmax[kChunk];   // list indices of c1, c2; 0xFFFFFFFF hmax: no affinity
-        uint32_t ch[kChunk];                    // list index chosen
+        alignas(16) uint32_t hit[kChunk][32 * J];
+        uint64_t cl[kChunk];      // cost x L
+        uint64_t w0[32 * J];      // loads at the chunk's start
+        uint64_t wk[kChunk];      // work that the request adds to the chosen instance
+        uint32_t hmax[kChunk];    // 0xFFFFFFFF: no affinity
+        uint32_t ch[kChunk];      // list index chosen
     };
     static size_t smem(uint32_t M) { return 32 * J * 20 + (size_t(M) * 2 + 15) / 16 * 16 + 3 * sizeof(Stage); }
 };
@@ -501,27 +508,83 @@ __global__ void __launch_bounds__(GlobalPipe<J>::kThreads) k_choice_all(DevState
 
     auto stage = [&](uint32_t buf, uint32_t k, uint32_t m, uint32_t base) {
         Stage &S = SB[buf];
-        for (uint32_t rr = k >> 5; rr < m; rr += kGlobalStageThreads / 32) {   // a warp per request
-            const uint32_t r = base + rr, L = d.r_L[r];
-            const uint32_t *ha = d.h_all + uint64_t(r) * d.M;
-            uint32_t h[J], hmax = 0;
+        constexpr uint32_t kWarps = kGlobalStageThreads / 32, G = 16 / J;   // a warp takes G requests' loads at a time
+        for (uint32_t q = k >> 5; q < m; q += kWarps * G) {
+            uint32_t h[G][J], L[G];
+#pragma unroll
+            for (uint32_t g = 0; g < G; ++g) {
+                const uint32_t rr = q + g * kWarps;
+                const uint32_t *ha = d.h_all + uint64_t(base + rr) * d.M;
+                L[g] = rr < m ? d.r_L[base + rr] : 0;
+#pragma unroll
+                for (uint32_t j = 0; j < J; ++j) {
+                    const uint32_t x = j * 32 + lane;
+                    h[g][j] = rr < m && x < nl ? ha[live[x]] : 0;
+                }
+            }
+#pragma unroll
+            for (uint32_t g = 0; g < G; ++g) {
+                const uint32_t rr = q + g * kWarps;
+                if (rr >= m) break;
+                uint32_t hmax = 0;
+#pragma unroll
+                for (uint32_t j = 0; j < J; ++j) {
+                    S.hit[rr][j * 32 + lane] = h[g][j];
+                    hmax = max(hmax, h[g][j]);
+                }
+                if (rule == DM_RULE_PREBLE) hmax = __reduce_max_sync(0xffffffffu, hmax);
+                if (lane == 0) {
+                    S.cl[rr] = cost * L[g];
+                    S.hmax[rr] = rule == DM_RULE_PREBLE && 2ull * hmax > L[g] ? hmax : 0xFFFFFFFFu;
+                }
+            }
+        }
+    };
+
+    // one chunk with 31-bit loads and work; w: this lane's loads, moved on
+    constexpr uint32_t kNever = 0x80000000u;
+    auto decide32 = [&](auto kind, Stage &S, uint32_t m, uint32_t (&w)[J]) {
+        constexpr uint32_t kRule = decltype(kind)::value;
+        struct alignas(J >= 4 ? 16 : 8) Hits {
+            uint32_t v[J];
+        };
+        const uint32_t c32 = (uint32_t)cost;
+        // the next request's staged values, read while this one is decided
+        Hits h = *reinterpret_cast<const Hits *>(&S.hit[0][lane * J]);
+        uint32_t cl = (uint32_t)S.cl[0], hm = S.hmax[0];
+        for (uint32_t rr = 0; rr < m; ++rr) {
+            uint32_t u[J], add[J];   // its work on each instance; what its key adds to the load
+            bool out[J];             // Preble's affinity leaves the instance out
 #pragma unroll
             for (uint32_t j = 0; j < J; ++j) {
-                const uint32_t x = j * 32 + lane;
-                h[j] = x < nl ? ha[live[x]] : 0;
+                u[j] = cl - c32 * h.v[j];
+                out[j] = kRule == DM_RULE_PREBLE && hm != 0xFFFFFFFFu && h.v[j] != hm;
+                add[j] = kRule == DM_RULE_LEAST_LOADED || (kRule == DM_RULE_PREBLE && hm != 0xFFFFFFFFu) ? 0u : u[j];
             }
+            const uint32_t nx = min(rr + 1, m - 1);
+            h = *reinterpret_cast<const Hits *>(&S.hit[nx][lane * J]);
+            cl = (uint32_t)S.cl[nx];
+            hm = S.hmax[nx];
+            uint32_t bk[J], bj[J];
 #pragma unroll
             for (uint32_t j = 0; j < J; ++j) {
-                S.hit[rr][j * 32 + lane] = h[j];
-                hmax = max(hmax, h[j]);
+                bk[j] = out[j] ? 0xFFFFFFFFu : w[j] + add[j];
+                bj[j] = j;
             }
-            hmax = __reduce_max_sync(0xffffffffu, hmax);
-            if (lane == 0) {
-                S.cl[rr] = cost * L;
-                S.hmax[rr] = rule == DM_RULE_PREBLE && 2ull * hmax > L ? hmax : 0xFFFFFFFFu;
-                S.ci[0][rr] = inv[d.r_c1[r]];
-                S.ci[1][rr] = inv[d.r_c2[r]];
-            }
+#pragma unroll
+            for (uint32_t s = 1; s < J; s *= 2)   // ties: the lower index
+#pragma unroll
+                for (uint32_t j = 0; j + s < J; j += 2 * s) {
+                    const bool less = bk[j + s] < bk[j];
+                    bk[j] = less ? bk[j + s] : bk[j];
+                    bj[j] = less ? bj[j + s] : bj[j];
+                }
+            const uint32_t kmin = __reduce_min_sync(0xffffffffu, bk[0]);
+            const uint32_t eq = __ballot_sync(0xffffffffu, bk[0] == kmin);
+            const uint32_t won = eq & (0u - eq) & (1u << lane) ? bj[0] : J;   // the lowest lane's index
+#pragma unroll
+            for (uint32_t j = 0; j < J; ++j) w[j] += won == j ? u[j] : 0u;
+            if (won < J) S.ch[rr] = lane * J + won;
         }
     };
 
@@ -535,6 +598,7 @@ __global__ void __launch_bounds__(GlobalPipe<J>::kThreads) k_choice_all(DevState
             const uint32_t x = lane * J + j;
             w64[j] = x < nl ? W[x] : ~0ull;
             if (x < nl) {
+                S.w0[x] = w64[j];
                 lo = min(lo, w64[j]);
                 hi = max(hi, w64[j]);
             }
@@ -550,56 +614,19 @@ __global__ void __launch_bounds__(GlobalPipe<J>::kThreads) k_choice_all(DevState
             work += shfl_xor_u64(work, x);
         }
         small = __all_sync(0xffffffffu, small);
-        constexpr uint32_t kNever = 0x80000000u;   // above every key that may win
         if (small && hi - lo < kNever && work < kNever - (hi - lo)) {
-            uint32_t w[J];
+            uint32_t w[J];   // past the list: above every key that may win
 #pragma unroll
-            for (uint32_t j = 0; j < J; ++j) w[j] = lane * J + j < nl ? (uint32_t)(w64[j] - lo) : 0xFFFFFFFFu;
-            const uint32_t c32 = (uint32_t)cost;
-            // each request's keys less the loads, read one request ahead
-            uint32_t u[J], add[J];
-            auto read = [&](uint32_t rr) {
-                const uint32_t cl = (uint32_t)S.cl[rr], hm = S.hmax[rr];
+            for (uint32_t j = 0; j < J; ++j) w[j] = lane * J + j < nl ? (uint32_t)(w64[j] - lo) : kNever;
+            if (rule == DM_RULE_MIN_TTFT) decide32(std::integral_constant<uint32_t, DM_RULE_MIN_TTFT>{}, S, m, w);
+            else if (rule == DM_RULE_LEAST_LOADED)
+                decide32(std::integral_constant<uint32_t, DM_RULE_LEAST_LOADED>{}, S, m, w);
+            else decide32(std::integral_constant<uint32_t, DM_RULE_PREBLE>{}, S, m, w);
 #pragma unroll
-                for (uint32_t j = 0; j < J; ++j) {
-                    const uint32_t h = S.hit[rr][lane * J + j];
-                    u[j] = cl - c32 * h;
-                    add[j] = rule == DM_RULE_LEAST_LOADED ? 0u : hm == 0xFFFFFFFFu ? u[j] : h == hm ? 0u : kNever;
-                    if (lane * J + j >= nl) add[j] = 0;   // w stays above every key
-                }
-            };
-            read(0);
-            for (uint32_t rr = 0; rr < m; ++rr) {
-                const uint64_t wc = lane < 2 ? Wv[S.ci[lane & 1][rr]] : 0;   // as this request finds them
-                __syncwarp();
-                uint32_t bk = w[0] + add[0], bu = u[0], bj = 0, bw = w[0];
-#pragma unroll
-                for (uint32_t j = 1; j < J; ++j) {
-                    const uint32_t key = w[j] + add[j];
-                    const bool less = key < bk;
-                    bk = less ? key : bk;
-                    bu = less ? u[j] : bu;
-                    bw = less ? w[j] : bw;
-                    bj = less ? j : bj;
-                }
-                const uint32_t kmin = __reduce_min_sync(0xffffffffu, bk);
-                const uint32_t eq = __ballot_sync(0xffffffffu, bk == kmin);
-                const bool win = bk == kmin && (eq & ((1u << lane) - 1u)) == 0;
-                const uint32_t nw = bw + bu;
-#pragma unroll
-                for (uint32_t j = 0; j < J; ++j) w[j] = win && bj == j ? nw : w[j];
-                if (win) {
-                    Wv[lane * J + bj] = lo + nw;
-                    S.wch[rr] = lo + nw;
-                    S.ch[rr] = lane * J + bj;
-                }
-                if (rr + 1 < m) read(rr + 1);
-                if (lane < 2) S.t[lane][rr] = wc;
-                __syncwarp();
-            }
+            for (uint32_t j = 0; j < J; ++j)
+                if (lane * J + j < nl) W[lane * J + j] = lo + w[j];
         } else {
             for (uint32_t rr = 0; rr < m; ++rr) {
-                const uint64_t wc = lane < 2 ? Wv[S.ci[lane & 1][rr]] : 0;
                 const uint64_t cl = S.cl[rr];
                 const uint32_t hm = S.hmax[rr];
                 // smallest (key, list index): three 32-bit reductions give the exact pair
@@ -624,28 +651,39 @@ __global__ void __launch_bounds__(GlobalPipe<J>::kThreads) k_choice_all(DevState
                     __reduce_min_sync(0xffffffffu, bk == ((uint64_t(khi) << 32) | klo) ? bx : 0xFFFFFFFFu);
                 __syncwarp();
                 if (lane == 0) {
-                    const uint64_t nw = Wv[x] + cl - cost * S.hit[rr][x];
-                    Wv[x] = nw;
-                    S.wch[rr] = nw;
+                    Wv[x] = Wv[x] + cl - cost * S.hit[rr][x];
                     S.ch[rr] = x;
                 }
-                if (lane < 2) S.t[lane][rr] = wc;
                 __syncwarp();
             }
         }
     };
 
     auto emit = [&](uint32_t buf, uint32_t k, uint32_t m, uint32_t base) {
-        const Stage &S = SB[buf];
+        Stage &S = SB[buf];
         const bool valid = k < m;
         const uint32_t r = base + k, x = valid ? S.ch[k] : 0;
-        const uint32_t nbr = valid ? d.r_nblk[r] : 0;
+        const uint32_t nbr = valid ? d.r_nblk[r] : 0, h = valid ? S.hit[k][x] : 0;
+        const uint64_t wk = valid ? S.cl[k] - cost * h : 0;
+        if (valid) S.wk[k] = wk;
+        // (its barriers also order the chunk's wk before the sums below)
         const uint64_t pt =
             record_place<kChunk>(PT, x, (uint64_t(nbr) << 32) + 1, valid, k / 32, (m + 31) / 32, lane);
         if (!valid) return;
-        const uint32_t ch = live[x], h = S.hit[k][x], L = d.r_L[r];
+        const uint32_t ch = live[x], L = d.r_L[r], c1 = d.r_c1[r], c2 = d.r_c2[r];
         const uint32_t h1 = hit_tokens(d.r_m1[r], nbr, d.B), h2 = hit_tokens(d.r_m2[r], nbr, d.B);
-        const uint64_t t1 = S.t[0][k] + cost * (L - h1), t2 = S.t[1][k] + cost * (L - h2);
+        // the loads as the request found them
+        const uint32_t x1 = inv[c1], x2 = inv[c2];
+        uint64_t wc = S.w0[x], w1 = S.w0[x1], w2 = S.w0[x2];
+        for (uint32_t q = 0; q < (k | 31u); ++q) {
+            if (q >= k) continue;
+            const uint32_t cq = S.ch[q];
+            const uint64_t wq = S.wk[q];
+            wc += cq == x ? wq : 0;
+            w1 += cq == x1 ? wq : 0;
+            w2 += cq == x2 ? wq : 0;
+        }
+        const uint64_t t1 = w1 + cost * (L - h1), t2 = w2 + cost * (L - h2);
         o.ttft1[r] = t1;
         o.ttft2[r] = t2;
         o.chosen[r] = ch;
@@ -654,7 +692,7 @@ __global__ void __launch_bounds__(GlobalPipe<J>::kThreads) k_choice_all(DevState
         d.r_touchoff[r] = pt >> 32;
         ms.tokens += L;
         ms.hits += h;
-        ms.est += S.wch[k] <= slo;
+        ms.est += wc + wk <= slo;
         if (t1 > slo && t2 > slo) d.info->both_over = 1;
         const uint32_t slot = (uint32_t)pt;
         if (slot - d.q_head[ch] >= d.Q) {
@@ -663,10 +701,10 @@ __global__ void __launch_bounds__(GlobalPipe<J>::kThreads) k_choice_all(DevState
         }
         QEntry e;
         e.seq = seq0 + r;
-        e.work = e.remaining = cost * (L - h);
+        e.work = e.remaining = wk;
         e.L = L;
-        e.c1 = d.r_c1[r];
-        e.c2 = d.r_c2[r];
+        e.c1 = c1;
+        e.c2 = c2;
         e.h1 = h1;
         e.h2 = h2;
         e.moved = 0;
