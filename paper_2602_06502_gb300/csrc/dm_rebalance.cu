@@ -13,6 +13,11 @@
 // is still hot, the benefit (re-evaluated with the current W_j) is positive
 // and TTFT_{r,j} < SLO.  Moved requests leave a tombstone (zero work) in the
 // source queue and are appended to the target queue.
+//
+// Most hotspots have no request that could move (256 instances, 4,096 prompts
+// a batch: 31-38 hotspots, 1-9 moves).  So a warp per hotspot first looks for
+// one under the loads at the call's start, all hotspots at once, and only the
+// hotspots that might move one are visited (scan_hotspot).
 #include "dm_internal.cuh"
 
 namespace dm {
@@ -136,7 +141,7 @@ struct RbChunk {
 };
 
 // Dynamic shared memory layout: per instance W (u64), queue tails (u32),
-// hot list (u32), state (u8, padded); then the chunk staging; then the sort
+// hot list (u32), state and flags (u8, padded); then the chunk staging; then the sort
 // arrays (key u64, seq u64, ttft u64, pos u32) of up to `sort_cap` candidates.
 __host__ __device__ inline size_t rb_inst_bytes(uint32_t M) { return (size_t(M) * 17 + 15) / 16 * 16; }
 __host__ __device__ inline size_t rb_sort_bytes(uint32_t cap) { return size_t(cap) * 28; }
@@ -166,6 +171,58 @@ __device__ void bitonic_sort(uint64_t *key, uint64_t *seq, uint64_t *tt, uint32_
     }
 }
 
+// Whether a request queued on hotspot i could move, from the loads at the
+// call's start.  Visits before i's change this only through the loads of i's
+// targets: work moved to a target makes a move to it less likely, so a hotspot
+// without a candidate now has none at its turn unless an earlier hotspot that
+// it would move to has given work away.  Returns whether a request passes the
+// move test now; *later: bit (id & 63) of each earlier hotspot to which a
+// request would move if nothing were queued there.  Whole warp; the next 32
+// entries are loaded while these are tested.
+// Per-instance byte: the instance's state and two flags of this call.
+constexpr uint8_t kStMask = 0x3F, kStHot = 0x80, kStIdle = 0x40;   // hotspot; hotspot with nothing to move now
+constexpr uint32_t kLater = 128;   // hotspots (by rank) whose `later` is kept; those after it: any
+struct ScanEntry {
+    uint64_t work, remaining;
+    uint32_t L, c1, c2, h1, h2, moved;
+};
+__device__ __forceinline__ ScanEntry scan_entry(const QEntry *q, uint32_t mask, uint32_t p, bool valid) {
+    ScanEntry s{};
+    if (valid) {
+        const QEntry &e = q[p & mask];
+        s = ScanEntry{e.work, e.remaining, e.L, e.c1, e.c2, e.h1, e.h2, e.moved};
+    }
+    return s;
+}
+__device__ bool scan_hotspot(const DevState &d, uint32_t i, uint32_t tail, uint32_t call, const uint64_t *W,
+                             const uint8_t *st, int lane, uint64_t *later) {
+    const QEntry *qi = d.q + uint64_t(i) * d.Q;
+    const uint32_t head = d.q_head[i], len = tail - head;
+    uint64_t ahead = 0, lt = 0;
+    bool now = false;
+    ScanEntry nx = scan_entry(qi, d.Q - 1, head + lane, (uint32_t)lane < len);
+    for (uint32_t p0 = 0; p0 < len; p0 += 32) {
+        const ScanEntry e = nx;
+        const bool valid = p0 + lane < len;
+        nx = scan_entry(qi, d.Q - 1, head + p0 + 32 + lane, p0 + 32 + lane < len);
+        const uint64_t inc = warp_incl_scan(e.remaining, lane);
+        if (valid && e.moved != kTomb && e.moved != call && e.remaining == e.work) {
+            const uint64_t ttft_i = ahead + inc;
+            const uint32_t j = e.c1 == i ? e.c2 : e.c1;
+            const uint64_t own = d.cost * (e.L - (j == e.c1 ? e.h1 : e.h2));
+            const uint64_t ttft_j = W[j] + own;
+            if ((int64_t)(ttft_i - ttft_j) > 0 && ttft_j < d.slo) now = true;
+            const bool earlier = (st[j] & kStHot) && (W[j] > W[i] || (W[j] == W[i] && j < i));
+            if (earlier && (int64_t)(ttft_i - own) > 0 && own < d.slo) lt |= 1ull << (j & 63);
+        }
+        ahead += shfl_u64(inc, 31);
+    }
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) lt |= shfl_xor_u64(lt, o);
+    *later = lt;
+    return __any_sync(0xffffffffu, now);
+}
+
 // Single CTA of 1024 threads.
 __global__ void __launch_bounds__(1024) k_rebalance(DevState d, uint32_t n, uint64_t seq0, uint32_t call,
                                                     dm_migration *out, uint32_t cap, uint32_t *n_out,
@@ -174,8 +231,8 @@ __global__ void __launch_bounds__(1024) k_rebalance(DevState d, uint32_t n, uint
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint32_t s_w[33];
     __shared__ uint64_t s_u[33];
-    __shared__ uint64_t s_sumW;
-    __shared__ uint32_t s_nhot, s_cnt, s_nmv, s_stop;
+    __shared__ uint64_t s_sumW, s_later[kLater];
+    __shared__ uint32_t s_cnt, s_nmv, s_stop;
     if (has_err(d.err)) return;
     const uint32_t M = d.M;
     uint64_t *W = reinterpret_cast<uint64_t *>(smem);
@@ -223,11 +280,25 @@ __global__ void __launch_bounds__(1024) k_rebalance(DevState d, uint32_t n, uint
             rk += (W[y] > W[x]) || (W[y] == W[x] && y < x);
         }
         hotl[rk] = x;
+        st[x] |= kStHot;
     }
-    if (threadIdx.x == 0) { s_sumW = sumW0; s_cnt = 0; s_nhot = nhot; }
+    if (threadIdx.x == 0) { s_sumW = sumW0; s_cnt = 0; }
     __syncthreads();
     const uint64_t cost = d.cost;
-    for (uint32_t hi = 0; hi < s_nhot; ++hi) {
+    for (uint32_t hi = threadIdx.x >> 5; hi < nhot && !fresh; hi += blockDim.x >> 5) {   // fresh hits are probed at the visit
+        const uint32_t i = hotl[hi];
+        uint64_t later;
+        const bool now = scan_hotspot(d, i, tails[i], call, W, st, threadIdx.x & 31, &later);
+        if ((threadIdx.x & 31) == 0) {
+            if (!now) st[i] |= kStIdle;
+            if (hi < kLater) s_later[hi] = later;
+        }
+    }
+    __syncthreads();
+    uint64_t gave = 0;   // bit (id & 63): hotspots that moved work away
+    for (uint32_t hi = 0; hi < nhot; ++hi) {
+        if ((st[hotl[hi]] & kStIdle) && ((hi < kLater ? s_later[hi] : ~0ull) & gave) == 0) continue;
+        const uint32_t cnt_before = s_cnt;
         const uint32_t i = hotl[hi];
         QEntry *qi = d.q + uint64_t(i) * d.Q;
         const uint32_t head = d.q_head[i], tail = tails[i];
@@ -249,7 +320,7 @@ __global__ void __launch_bounds__(1024) k_rebalance(DevState d, uint32_t n, uint
                 // probe the other candidate's index now, a warp per entry in
                 // turn; the pending batch's own entries keep their stored
                 // hit (no commit since their routing: the same probe)
-                const bool need = elig && st[jj] == 1 && !(e.seq >= seq0 && e.seq < seq0 + n);
+                const bool need = elig && (st[jj] & kStMask) == 1 && !(e.seq >= seq0 && e.seq < seq0 + n);
                 const int lane = threadIdx.x & 31;
                 for (uint32_t m = __ballot_sync(0xffffffffu, need); m; m &= m - 1) {
                     const int src = __ffs(m) - 1;
@@ -355,7 +426,7 @@ __global__ void __launch_bounds__(1024) k_rebalance(DevState d, uint32_t n, uint
                         break;
                     }
                     const uint32_t j = Ch.j[k];
-                    if (st[j] != 1) continue;
+                    if ((st[j] & kStMask) != 1) continue;
                     const uint64_t nw = Ch.new_work[k];
                     const uint64_t ttft_j = W[j] + nw;
                     if (!(Ch.ttft_i[k] > ttft_j && ttft_j < d.slo)) continue;
@@ -428,6 +499,7 @@ __global__ void __launch_bounds__(1024) k_rebalance(DevState d, uint32_t n, uint
             if (threadIdx.x == 0) s_cnt = cnt0 + s_nmv;
             __syncthreads();
         }
+        if (s_cnt != cnt_before) gave |= 1ull << (i & 63);
     }
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < M; i += blockDim.x) {
