@@ -460,6 +460,8 @@ __global__ void __launch_bounds__(kMtThreads) k_maint_c(DevState d, uint32_t n) 
 __device__ void commit_prep_cta(const DevState &d, uint32_t n, uint64_t *adv) {
     for (uint32_t i = threadIdx.x; i < d.M; i += blockDim.x) {
         const uint32_t fl = d.mt_flags[i];
+        const uint64_t live = min(d.live[i], d.C);   // the last commit's eviction left C
+        d.live[i] = live;
         if (fl & kFlagCompact) {
             Rec *a = d.logbuf[i];
             d.logbuf[i] = d.logbuf_alt[i];
@@ -477,7 +479,7 @@ __device__ void commit_prep_cta(const DevState &d, uint32_t n, uint64_t *adv) {
             d.pool[d.rb_slot[i]] = d.table[i];
             d.table[i] = d.table_alt[i];
             d.table_alt[i] = nullptr;
-            d.used[i] = d.live[i];
+            d.used[i] = live;
             atomicAdd(reinterpret_cast<unsigned long long *>(&d.maint_count[0]), 1ull);
         }
         adv[i] = d.log_adv[i];
@@ -801,8 +803,9 @@ __global__ void __cluster_dims__(kEvCluster, 1, 1) __launch_bounds__(kEvThreads)
     const uint32_t go = *cluster.map_shared_rank(&s_go, 0);
     const uint64_t lmask = d.logcap - 1;
     uint32_t slot = 0;
-    // the instances over capacity, in id order (every CTA builds the same
-    // list), dealt to the clusters in turn
+    // the instances over capacity, in id order, dealt to the clusters in turn.
+    // Every CTA builds the same list whenever it starts: nothing in this kernel
+    // writes live_i, which the next commit cuts to C
     uint32_t nev = 0;
     for (uint32_t base = 0; go && base < d.M; base += blockDim.x) {
         const uint32_t i = base + threadIdx.x;
@@ -906,12 +909,9 @@ __global__ void __cluster_dims__(kEvCluster, 1, 1) __launch_bounds__(kEvThreads)
             base += uint64_t(kEvThreads) * per * kEvCluster;
             front = min(base, tail);
         }
-        if (r == 0 && threadIdx.x == 0) {
-            if (remaining) {   // the log must cover every live key
-                set_err(d.err, DM_ERR_TIMEOUT);
-                d.log_front[i] = front;
-            }
-            d.live[i] = d.C;
+        if (r == 0 && threadIdx.x == 0 && remaining) {   // the log must cover every live key
+            set_err(d.err, DM_ERR_TIMEOUT);
+            d.log_front[i] = front;
         }
     }
     cluster.sync();   // no CTA leaves while another may still read its shared memory
