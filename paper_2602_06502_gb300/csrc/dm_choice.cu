@@ -8,9 +8,9 @@
 // Choice between two candidates (DualMap's rule and the pair variants):
 // the decision for a request depends on the loads left by every earlier
 // request of the batch that shares one of its candidates.  One CTA keeps W
-// in shared memory; one warp decides 32 requests at a time in dependency
-// rounds (a request waits only for earlier requests of the window sharing
-// an instance with it); everything that does not depend on W is precomputed
+// in shared memory; one warp decides 32 requests at a time, level by level (a
+// request follows only the earlier requests of the window that share an
+// instance with it); everything that does not depend on W is precomputed
 // in parallel, and queue writes and outputs are emitted in parallel
 // afterwards.
 //
@@ -99,75 +99,98 @@ __device__ void finish_metrics(const DevState &d, uint32_t n, MetricSums ms, uns
 // one another through the same pair.  So one warp does nothing but decide,
 // and everything else is kept out of its way:
 //   stage   a warp per window of 32 requests loads the requests and finds
-//           each one's level, 1 + the largest level of the earlier requests
-//           of its window that share an instance with it.  The levels depend
-//           on the candidates alone, so they are known before any decision;
-//   decide  warp 0, window by window, level by level: requests of one level
-//           share no instance, so reading W and writing W[choice] for all of
-//           them at once equals arrival order exactly.  A level is two loads,
-//           a compare and a store in shared memory: no vote, no branch on
-//           what is done;
+//           which request of its window each one follows on each of its
+//           candidates, and its level, one more than the largest of those.
+//           Both depend on the candidates alone, so they are known before
+//           any decision;
+//   decide  warp 0, window by window, level by level.  Loads that fit 32 bits
+//           pass from request to request (registers and shuffles for two
+//           candidates, a shared-memory row per lane for d); every lane decides
+//           at every level, so nothing waits or branches, and a request is
+//           right from its level on.  Larger loads stay in shared memory: the
+//           requests of one level share no instance, so reading W and writing
+//           W[choice] for all of them at once equals arrival order exactly;
 //   emit    a warp per window places the requests among their instances'
 //           records and queue entries and writes every output.
 // Chunk t is staged while chunk t - 1 is decided and chunk t - 2 emitted,
-// over three staging buffers.  Measured (GB300, a routed and committed pass
-// of 4,096 agent prompts): 311 us when windows were decided in rounds found
-// by votes, by the warp that also kept the record counters, with staging,
-// deciding and emitting one after the other; 255 us so.  The d-candidate
-// choice, one thread from global memory before: 5,360 and 577 us (d = 4).
+// over three staging buffers.  Measured (GB300, kernel time for 4,096 agent
+// prompts, two and four candidates): 191 and 5,200 us with rounds found by
+// votes and with one thread; 123 and 404 us when the deciding warp read and
+// wrote 64-bit loads in shared memory at every level (136 and 400 cycles a
+// level, 780 a window); 88 and 175 us so (84 cycles a level, 470 a window).
 constexpr uint8_t kNoLevel = 255;
 
+// The deciding warp has its SM sub-partition to itself (warps are dealt to the
+// four by their number): every fourth warp only meets the barriers.  Beside
+// emitting or staging warps the same chain ran 10-20 % longer (a pass of 4,096
+// agent prompts 250 and 230 us, min TTFT over 64 instances 680 and 615).
 template <uint32_t kChunk, uint32_t kStageThreads = kChunk>
 struct Pipe {
-    static constexpr uint32_t kThreads = 32 + kChunk + kStageThreads;   // warp 0, the emitting and staging warps
+    static constexpr uint32_t kWorkers = (kChunk + kStageThreads) / 32;   // the emitting, then the staging warps
+    static constexpr uint32_t kThreads = 32 * (1 + kWorkers + (kWorkers - 1) / 3);
 };
 
 // stage(buffer, k, m, base), decide(buffer, m), emit(buffer, k, m, base): k
 // the thread's number among its role's (an emitting thread's request of the
 // chunk; whole windows call, k >= m past the batch's end), m the chunk's
 // requests, base its first request.
-template <uint32_t kChunk, class StageF, class DecideF, class EmitF>
+template <uint32_t kChunk, uint32_t kStageThreads, class StageF, class DecideF, class EmitF>
 __device__ __forceinline__ void choice_pipeline(uint32_t n, StageF stage, DecideF decide, EmitF emit) {
-    const uint32_t nc = (n + kChunk - 1) / kChunk, tid = threadIdx.x;
+    const uint32_t nc = (n + kChunk - 1) / kChunk, wid = threadIdx.x >> 5;
+    const uint32_t w = 32 * (wid - 1 - wid / 4) + (threadIdx.x & 31);   // number among the workers (wid % 4 != 0)
     for (uint32_t t = 0; t < nc + 2; ++t) {
-        if (tid < 32) {
+        if (wid == 0) {
             if (t >= 1 && t <= nc) decide((t - 1) % 3, min(kChunk, n - (t - 1) * kChunk));
-        } else if (tid < 32 + kChunk) {
-            if (t >= 2) emit((t - 2) % 3, tid - 32, min(kChunk, n - (t - 2) * kChunk), (t - 2) * kChunk);
-        } else {
-            if (t < nc) stage(t % 3, tid - 32 - kChunk, min(kChunk, n - t * kChunk), t * kChunk);
+        } else if (wid % 4 == 0) {
+        } else if (w < kChunk) {
+            if (t >= 2) emit((t - 2) % 3, w, min(kChunk, n - (t - 2) * kChunk), (t - 2) * kChunk);
+        } else if (w < kChunk + kStageThreads) {
+            if (t < nc) stage(t % 3, w - kChunk, min(kChunk, n - t * kChunk), t * kChunk);
         }
         __syncthreads();
     }
 }
 
-// Level of this lane's request in its window (0 first; valid: there is one),
-// from the candidates of all lanes packed in c (kWords words, two 16-bit ids
-// each; unused halves 0xFFFF).  Whole warp; returns also the window's number
-// of levels.
-template <int kWords>
-__device__ __forceinline__ uint32_t window_levels(const uint32_t (&c)[kWords], bool valid, int lane,
-                                                  uint32_t &nlev) {
-    uint32_t lev = 0;
-    const uint32_t vm = __ballot_sync(0xffffffffu, valid);
-    for (int j = 0; j < 31; ++j) {
-        uint32_t o[kWords];
-        bool hit = false;
+// How the requests of a window follow one another: for each of this lane's ND
+// candidates c (0xFFFFFFFF past the batch's end; distinct instances) the latest
+// earlier request of the window that names the same instance, as from[f] =
+// its lane * kStride + its candidate's number (kNone: none), and in the result
+// bit f whether no later one does.  lev: the request's level, one more than
+// the largest of those it follows (0: none); nlev: the window's number of
+// levels.  Whole warp.
+constexpr uint32_t kNone = 0xFFFFFFFFu;
+template <uint32_t ND, uint32_t kStride>
+__device__ __forceinline__ uint32_t window_links(const uint32_t (&c)[ND], bool valid, int lane, uint32_t (&from)[ND],
+                                                 uint32_t &lev, uint32_t &nlev) {
+    uint32_t later = 0;
 #pragma unroll
-        for (int x = 0; x < kWords; ++x) o[x] = __shfl_sync(0xffffffffu, c[x], j);
+    for (uint32_t f = 0; f < ND; ++f) from[f] = kNone;
+#pragma unroll 4
+    for (int j = 0; j < 32; ++j) {
+        const bool before = j < lane, after = j > lane;
 #pragma unroll
-        for (int x = 0; x < kWords; ++x) {
+        for (uint32_t y = 0; y < ND; ++y) {
+            const uint32_t o = __shfl_sync(0xffffffffu, c[y], j);
 #pragma unroll
-            for (int y = 0; y < kWords; ++y) {   // a set half-word of vcmpeq: an id both name
-                const uint32_t sw = __byte_perm(o[y], 0, 0x1032);
-                hit |= ((__vcmpeq2(c[x], o[y]) | __vcmpeq2(c[x], sw)) & ~__vcmpeq2(c[x], 0xFFFFFFFFu)) != 0;
+            for (uint32_t f = 0; f < ND; ++f) {
+                from[f] = o == c[f] && before ? j * kStride + y : from[f];
+                later |= o == c[f] && after ? 1u << f : 0u;
             }
         }
-        const uint32_t lj = __shfl_sync(0xffffffffu, lev, j);
-        if (hit && lane > j && ((vm >> j) & 1u)) lev = max(lev, lj + 1);
+    }
+    lev = 0;
+    for (bool more = true; more;) {
+        uint32_t nl = 0;
+#pragma unroll
+        for (uint32_t f = 0; f < ND; ++f) {
+            const uint32_t x = __shfl_sync(0xffffffffu, lev, from[f] / kStride);   // (kNone: any lane)
+            nl = max(nl, valid && from[f] != kNone ? x + 1 : 0);
+        }
+        more = __any_sync(0xffffffffu, nl != lev);
+        lev = nl;
     }
     nlev = __reduce_max_sync(0xffffffffu, valid ? lev + 1 : 0);
-    return lev;
+    return valid ? ~later & ((1u << ND) - 1u) : 0;
 }
 
 // Each request is staged as (a, b): a = the candidate with more cached
@@ -179,14 +202,24 @@ __device__ __forceinline__ uint32_t window_levels(const uint32_t (&c)[kWords], b
 // W_a > thr and (k_b < k_a or (k_b == k_a and tieb)), with k = W (+ u when
 // the rule compares TTFTs) and tieb set where a tie goes to b (= c1).
 constexpr uint32_t kChoiceChunk = 256;
+constexpr uint64_t kSmall = 1ull << 30;   // loads below it are decided in 32 bits
 struct ChoiceStage {
     uint64_t ua[kChoiceChunk], ub[kChoiceChunk];
     int64_t thr[kChoiceChunk];
     uint64_t Wa[kChoiceChunk], Wb[kChoiceChunk];
     uint32_t ab[kChoiceChunk];     // a | b << 14 | (a is c2) << 28 | (hits differ) << 29 | tieb << 30 | addu << 31
+    // the same for a decision in 32 bits: a | b << 16, link, low words of ua and ub; thr (INT32_MAX at most) and lead
+    // (pair rules: choose b iff W_b - W_a < lead and W_a > thr)
+    uint4 rec[kChoiceChunk];
+    int2 lim[kChoiceChunk];
+    uint64_t wsum[kChoiceChunk / 32];   // per window: sum of the larger of both works (each kSmall at most)
     uint32_t nlev[kChoiceChunk / 32];
     uint8_t lev[kChoiceChunk], pickb[kChoiceChunk];
 };
+
+// link: bits 0-4 the lane that the request follows on a, bit 5 set: as that
+// lane's b, bit 6: there is one, bit 7: no later request of the window names a;
+// bits 8-15 the same for b; from bit 16 on the window's number of levels.
 
 // W and PT (8 bytes each) per instance, then the staging buffers.
 size_t choice_smem(uint32_t M) { return size_t(M) * 16 + 3 * sizeof(ChoiceStage); }
@@ -197,7 +230,7 @@ size_t choice_smem(uint32_t M) { return size_t(M) * 16 + 3 * sizeof(ChoiceStage)
 // Bound: about 1,250 dependent levels on an agent batch (4,096 requests, 64
 // instances, 200 templates).
 template <bool kPairRules>
-__global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads) k_choice(DevState d, dm_route_out o, uint32_t n,
+__global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads, 1) k_choice(DevState d, dm_route_out o, uint32_t n,
                                                                          uint64_t seq0, uint64_t t_batch) {
     pdl_enter();
     extern __shared__ __align__(16) unsigned char smem[];
@@ -210,7 +243,7 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads) k_choice(DevStat
     uint64_t *PT = W + d.M;
     ChoiceStage *const SB = reinterpret_cast<ChoiceStage *>(PT + d.M);
     const int lane = threadIdx.x & 31;
-    uint32_t live_bits = 0;   // bit k: instance threadIdx.x + k * blockDim.x is live (M <= 16 * 544)
+    uint32_t live_bits = 0;   // bit k: instance threadIdx.x + k * blockDim.x is live (M <= 16 * 704)
     for (uint32_t i = threadIdx.x, k = 0; i < d.M; i += blockDim.x, ++k) {
         W[i] = d.W[i];
         PT[i] = d.q_tail[i];
@@ -224,7 +257,8 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads) k_choice(DevStat
         if ((k & ~31u) >= m) return;   // no request in this window
         ChoiceStage &S = SB[buf];
         const bool valid = k < m;
-        uint32_t ids[1] = {0xFFFFFFFFu};
+        uint32_t ids[2] = {kNone, kNone}, u32[2] = {0, 0};
+        uint64_t most = 0;
         if (valid) {
             const uint32_t r = base + k;
             const uint32_t L = d.r_L[r], nblk = d.r_nblk[r];
@@ -254,16 +288,102 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads) k_choice(DevStat
             S.thr[k] = thr;
             S.ab[k] = (a2 ? c2 : c1) | ((a2 ? c1 : c2) << 14) | (uint32_t(a2) << 28) | (uint32_t(differ) << 29) |
                       (uint32_t(tieb) << 30) | (uint32_t(addu) << 31);
-            ids[0] = c1 | c2 << 16;
+            ids[0] = a2 ? c2 : c1;
+            ids[1] = a2 ? c1 : c2;
+            u32[0] = (uint32_t)ua;
+            u32[1] = (uint32_t)ub;
+            S.lim[k] = make_int2((int32_t)min(thr, (int64_t)INT32_MAX),
+                                 (addu ? (int32_t)(u32[0] - u32[1]) : 0) + (tieb ? 1 : 0));
+            most = min(max(ua, ub), kSmall);
         }
-        uint32_t nlev;
-        const uint32_t lev = window_levels<1>(ids, valid, lane, nlev);
+        uint32_t lev, nlev, from[2];
+        const uint32_t last = window_links<2, 2>(ids, valid, lane, from, lev, nlev);
+        uint32_t link = nlev << 16;
+#pragma unroll
+        for (uint32_t f = 0; f < 2; ++f) {
+            const uint32_t x = valid && from[f] != kNone ? from[f] / 2 | (from[f] & 1u) << 5 | 1u << 6 : 0;
+            link |= (x | ((last >> f) & 1u) << 7) << (8 * f);
+        }
+        S.rec[k] = make_uint4(valid ? ids[0] | ids[1] << 16 : 0, link, u32[0], u32[1]);
         S.lev[k] = valid ? (uint8_t)lev : kNoLevel;
-        if (lane == 0) S.nlev[k / 32] = nlev;
+        most = warp_sum_u64(most);
+        if (lane == 0) {
+            S.nlev[k / 32] = nlev;
+            S.wsum[k / 32] = most;
+        }
+    };
+
+    // one chunk whose loads stay below 2^30.  Every lane decides its request at
+    // every level, from the loads that the requests it follows leave (the
+    // loads at the window's start where there is none), so a request is right
+    // from its level on and the whole window after nlev levels: no lane waits
+    // or branches.  A level is four shuffles and a dozen operations in
+    // registers.  The window's last request on an instance leaves its load in
+    // W; the next window's staged values are read meanwhile.
+    uint64_t bound = 0;   // no load exceeds it
+    bool first = true;
+    auto decide32 = [&](ChoiceStage &S, uint32_t m) {
+        volatile uint32_t *const W32 = reinterpret_cast<volatile uint32_t *>(W);   // low words; the high ones are 0
+        uint4 nr = S.rec[lane];
+        int2 nl = S.lim[lane];   // past the batch's end: unused
+        for (uint32_t w0 = 0; w0 < m; w0 += 32) {
+            const uint4 x = nr;
+            const int32_t thr = nl.x, lead = kPairRules ? nl.y : 0;
+            const uint32_t a = x.x & 0xFFFF, b = x.x >> 16, link = x.y;
+            const uint32_t nlev = __reduce_max_sync(0xffffffffu, link >> 16);   // uniform: the loop below has no divergence
+            uint32_t A = W32[2 * a], B = W32[2 * b];
+            const uint32_t kn = (w0 + 32 < m ? w0 + 32 : 0) + lane;
+            nr = S.rec[kn];
+            nl = S.lim[kn];
+            const int sa = link & 31, sb = (link >> 8) & 31;
+            // where A and B come from: that lane's a, that lane's b, or here
+            auto mask = [&](uint32_t bits, uint32_t is) { return (bits & 0x60u) == is ? ~0u : 0u; };
+            const uint32_t ma0 = mask(link, 0x40u), ma1 = mask(link, 0x60u);
+            const uint32_t mb0 = mask(link >> 8, 0x40u), mb1 = mask(link >> 8, 0x60u);
+            const uint32_t Ah = A & ~(ma0 | ma1), Bh = B & ~(mb0 | mb1);
+            int32_t pb;   // all ones: b
+            uint32_t oA, oB;
+            auto step = [&] {
+                pb = ((int32_t)(B - A - lead) & (thr - (int32_t)A)) >> 31;
+                oA = A + (x.z & ~pb);
+                oB = B + (x.w & pb);
+            };
+            auto level = [&] {
+                const uint32_t A0 = __shfl_sync(0xffffffffu, oA, sa), A1 = __shfl_sync(0xffffffffu, oB, sa);
+                const uint32_t B0 = __shfl_sync(0xffffffffu, oA, sb), B1 = __shfl_sync(0xffffffffu, oB, sb);
+                A = (A0 & ma0) | Ah | (A1 & ma1);
+                B = (B0 & mb0) | Bh | (B1 & mb1);
+                step();
+            };
+            step();
+#pragma unroll 1
+            for (uint32_t l = 1; l < nlev; l += 2) {   // a level more than there are changes nothing
+                level();
+                level();
+            }
+            if (link & 0x80u) W32[2 * a] = oA;
+            if (link & 0x8000u) W32[2 * b] = oB;
+            __syncwarp();
+            const uint32_t k = w0 + lane;
+            S.Wa[k] = A;
+            S.Wb[k] = B;
+            S.pickb[k] = pb != 0;
+        }
     };
 
     auto decide = [&](uint32_t buf, uint32_t m) {
         ChoiceStage &S = SB[buf];
+        if (first) {
+            for (uint32_t i = lane; i < d.M; i += 32) bound = max(bound, W[i]);
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) bound = max(bound, shfl_xor_u64(bound, o));
+            first = false;
+        }
+        bound = min(bound, kSmall) + warp_sum_u64((uint32_t)lane < (m + 31) / 32 ? S.wsum[lane] : 0);
+        if (bound < kSmall) {
+            decide32(S, m);
+            return;
+        }
         volatile uint64_t *const Wv = W;
         for (uint32_t w0 = 0; w0 < m; w0 += 32) {
             const uint32_t k = w0 + lane;
@@ -353,7 +473,7 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads) k_choice(DevStat
     };
 
     __syncthreads();
-    choice_pipeline<kChoiceChunk>(n, stage, decide, emit);
+    choice_pipeline<kChoiceChunk, kChoiceChunk>(n, stage, decide, emit);
     unsigned __int128 S1 = 0, S2 = 0;
     uint32_t cnt = 0;
     for (uint32_t i = threadIdx.x, k = 0; i < d.M; i += blockDim.x, ++k) {
@@ -442,8 +562,7 @@ __global__ void __launch_bounds__(kAllBlock) k_probe_all(DevState d, uint32_t n)
 // 4,096 agent prompts on 64 instances, min TTFT, GB300: 1,678 us with 64-bit
 // keys and loads in shared memory, three reductions a request, and staging
 // and emission between the chunks; 922 us when the deciding warp also read
-// and wrote the loads in shared memory for every request, 1,247 us a pass;
-// 680 us a pass so.
+// and wrote the loads in shared memory for every request; 302 us so.
 constexpr uint32_t kGlobalStageThreads = 256;
 template <uint32_t J>
 struct GlobalPipe {
@@ -461,7 +580,7 @@ struct GlobalPipe {
 };
 
 template <uint32_t J>
-__global__ void __launch_bounds__(GlobalPipe<J>::kThreads) k_choice_all(DevState d, dm_route_out o, uint32_t n,
+__global__ void __launch_bounds__(GlobalPipe<J>::kThreads, 1) k_choice_all(DevState d, dm_route_out o, uint32_t n,
                                                                         uint64_t seq0, uint64_t t_batch) {
     pdl_enter();
     using P = GlobalPipe<J>;
@@ -714,7 +833,7 @@ __global__ void __launch_bounds__(GlobalPipe<J>::kThreads) k_choice_all(DevState
         d.q[uint64_t(ch) * d.Q + (slot & (d.Q - 1))] = e;
     };
 
-    choice_pipeline<kChunk>(n, stage, decide, emit);
+    choice_pipeline<kChunk, kGlobalStageThreads>(n, stage, decide, emit);
     unsigned __int128 S1 = 0, S2 = 0;
     uint32_t cnt = 0;
     for (uint32_t i = threadIdx.x; i < d.M; i += blockDim.x) {
@@ -1079,8 +1198,17 @@ struct ChoiceStageD {
     uint16_t c[ND][kChunk];
     uint8_t most[kChunk];             // bit f: candidate f has the most hit tokens
     uint8_t lev[kChunk], pick[kChunk], over[kChunk];
+    uint64_t wsum[kChunk / 32];       // per window: sum of the largest works (each kSmallD at most)
+    uint32_t u32[ND][kChunk];         // low words of u
+    uint16_t from[ND][kChunk];        // word of the exchange rows that holds candidate f's load
+    uint8_t last[kChunk];             // bit f: no later request of the window names candidate f
     uint32_t nlev[kChunk / 32];
 };
+constexpr uint64_t kSmallD = 1ull << 28;   // loads below it are decided in 32 bits, a candidate's number beside them
+// Exchange rows: for each lane what its request leaves on its candidates, then
+// the loads it found at the window's start; twice, written and read in turn.
+constexpr uint32_t exchange_stride(uint32_t nd) { return nd > 4 ? 8 : nd > 2 ? 4 : nd; }
+constexpr uint32_t exchange_words(uint32_t nd) { return 2 * 32 * exchange_stride(nd); }   // of one of the two
 constexpr uint32_t choice_d_chunk(uint32_t nd) { return nd <= 4 ? 256 : 128; }   // three buffers beside 8,192 instances
 
 // DualMap's rule over ND candidates, in arrival order (the pipeline above),
@@ -1088,7 +1216,7 @@ constexpr uint32_t choice_d_chunk(uint32_t nd) { return nd <= 4 ? 256 : 128; }  
 // k_choice leaves them.  Dynamic shared memory: W and the packed (records
 // << 32 | queue tail) counter of every instance, then the staging buffers.
 template <uint32_t ND>
-__global__ void __launch_bounds__(Pipe<choice_d_chunk(ND)>::kThreads) k_choice_d(DevState d, dm_route_out_d o,
+__global__ void __launch_bounds__(Pipe<choice_d_chunk(ND)>::kThreads, 1) k_choice_d(DevState d, dm_route_out_d o,
                                                                                  uint32_t n, uint64_t seq0,
                                                                                  uint64_t t_batch) {
     pdl_enter();
@@ -1099,8 +1227,10 @@ __global__ void __launch_bounds__(Pipe<choice_d_chunk(ND)>::kThreads) k_choice_d
     uint64_t *W = reinterpret_cast<uint64_t *>(smem);
     uint64_t *PT = W + d.M;
     Stage *const SB = reinterpret_cast<Stage *>(PT + d.M);
+    constexpr uint32_t kStride = exchange_stride(ND);
+    __shared__ alignas(16) uint32_t X[2 * exchange_words(ND)];
     const int lane = threadIdx.x & 31;
-    uint32_t live_bits = 0;   // bit k: instance threadIdx.x + k * blockDim.x is live (M <= 32 * 288)
+    uint32_t live_bits = 0;   // bit k: instance threadIdx.x + k * blockDim.x is live (M <= 32 * 352)
     for (uint32_t i = threadIdx.x, k = 0; i < d.M; i += blockDim.x, ++k) {
         W[i] = d.W[i];
         PT[i] = d.q_tail[i];
@@ -1113,9 +1243,10 @@ __global__ void __launch_bounds__(Pipe<choice_d_chunk(ND)>::kThreads) k_choice_d
         if ((k & ~31u) >= m) return;   // no request in this window
         Stage &S = SB[buf];
         const bool valid = k < m;
-        uint32_t ids[(ND + 1) / 2];
+        uint32_t ids[ND];
 #pragma unroll
-        for (uint32_t x = 0; x < (ND + 1) / 2; ++x) ids[x] = 0xFFFFFFFFu;
+        for (uint32_t f = 0; f < ND; ++f) ids[f] = kNone;
+        uint64_t umax = 0;
         if (valid) {
             const uint32_t r = base + k, L = d.r_L[r];
             const uint32_t *c = d.rd_cand + uint64_t(r) * ND, *h = d.rd_hit + uint64_t(r) * ND;
@@ -1129,23 +1260,139 @@ __global__ void __launch_bounds__(Pipe<choice_d_chunk(ND)>::kThreads) k_choice_d
             uint32_t most = 0;
 #pragma unroll
             for (uint32_t f = 0; f < ND; ++f) {
-                S.c[f][k] = (uint16_t)cf[f];
                 S.u[f][k] = cost * (L - hf[f]);
+                S.u32[f][k] = (uint32_t)S.u[f][k];
+                umax = max(umax, cost * (L - hf[f]));
                 most |= uint32_t(hf[f] == hmax) << f;
-                ids[f / 2] = f & 1 ? (ids[f / 2] & 0xFFFFu) | cf[f] << 16 : 0xFFFF0000u | cf[f];
+                ids[f] = cf[f];
                 o.cand[uint64_t(r) * ND + f] = cf[f];
                 o.hit[uint64_t(r) * ND + f] = hf[f];
             }
             S.most[k] = (uint8_t)most;
         }
-        uint32_t nlev;
-        const uint32_t lev = window_levels<(ND + 1) / 2>(ids, valid, lane, nlev);
+        uint32_t lev, nlev, from[ND];
+        S.last[k] = (uint8_t)window_links<ND, kStride>(ids, valid, lane, from, lev, nlev);
         S.lev[k] = valid ? (uint8_t)lev : kNoLevel;
-        if (lane == 0) S.nlev[k / 32] = nlev;
+#pragma unroll
+        for (uint32_t f = 0; f < ND; ++f) {
+            S.c[f][k] = valid ? (uint16_t)ids[f] : 0;   // every lane of a window reads its loads
+            S.from[f][k] = (uint16_t)(valid && from[f] != kNone ? from[f] : (32 + lane) * kStride + f);
+        }
+        umax = warp_sum_u64(min(umax, kSmallD));
+        if (lane == 0) {
+            S.nlev[k / 32] = nlev;
+            S.wsum[k / 32] = umax;
+        }
+    };
+
+    // one chunk whose loads stay below 2^28, as in k_choice: every lane decides
+    // its request at every level.  The loads pass between the lanes through
+    // shared memory (a row per lane).  A candidate's key is its load and its
+    // number, so one minimum over the candidates gives the least loaded and
+    // the earlier ring on ties; the candidates with the most hit tokens have
+    // the same uncached work.
+    uint64_t bound = 0;   // no load exceeds it
+    bool first = true;
+    struct Win {
+        uint32_t nlev, most, last, c[ND], u[ND], from[ND];
+    };
+    auto window = [&](const Stage &S, uint32_t w0) {
+        const uint32_t k = w0 + lane;
+        Win x;
+        x.nlev = S.nlev[w0 / 32];
+        x.most = S.most[k];
+        x.last = S.last[k];
+#pragma unroll
+        for (uint32_t f = 0; f < ND; ++f) {
+            x.c[f] = S.c[f][k];
+            x.u[f] = S.u32[f][k];   // past the batch's end: unused
+            x.from[f] = S.from[f][k];
+        }
+        return x;
+    };
+    auto decide32 = [&](Stage &S, uint32_t m) {
+        volatile uint32_t *const W32 = reinterpret_cast<volatile uint32_t *>(W);   // low words; the high ones are 0
+        constexpr uint32_t kRow = exchange_words(ND);
+        Win nx = window(S, 0);
+        for (uint32_t w0 = 0; w0 < m; w0 += 32) {
+            const Win x = nx;
+            uint32_t w[ND];
+#pragma unroll
+            for (uint32_t f = 0; f < ND; ++f) {
+                w[f] = W32[2 * x.c[f]];
+                X[(32 + lane) * kStride + f] = w[f];
+                X[kRow + (32 + lane) * kStride + f] = w[f];
+            }
+            nx = window(S, w0 + 32 < m ? w0 + 32 : 0);
+            // a misses the SLO iff its key > late (never when all hits are equal)
+            uint32_t ua = 0, skip[ND];
+#pragma unroll
+            for (uint32_t f = 0; f < ND; ++f) {
+                const bool in = (x.most >> f) & 1u;
+                ua = in ? x.u[f] : ua;
+                skip[f] = in ? 0u : 0x7FFFFFFFu;
+            }
+            const int32_t late = x.most == (1u << ND) - 1u ? INT32_MAX
+                                 : ua > slo               ? -1
+                                                          : (int32_t)(min(slo - ua, kSmallD - 1) * 8 + 7);
+            uint32_t key, out[ND], row = 0;
+            int32_t over;   // all ones: a misses the SLO and some candidate has fewer hits
+            auto step = [&] {
+                uint32_t kf[ND], ka[ND], km[ND];
+#pragma unroll
+                for (uint32_t f = 0; f < ND; ++f) {
+                    kf[f] = km[f] = w[f] * 8 + f;
+                    ka[f] = kf[f] | skip[f];
+                }
+#pragma unroll
+                for (uint32_t s = 1; s < ND; s *= 2)
+#pragma unroll
+                    for (uint32_t f = 0; f + s < ND; f += 2 * s) {
+                        ka[f] = min(ka[f], ka[f + s]);
+                        km[f] = min(km[f], km[f + s]);
+                    }
+                over = (late - (int32_t)ka[0]) >> 31;
+                const int32_t move = over & ((int32_t)(km[0] - (ka[0] & ~7u)) >> 31);   // the least loaded is below a
+                key = ka[0] ^ ((ka[0] ^ km[0]) & (uint32_t)move);
+#pragma unroll
+                for (uint32_t f = 0; f < ND; ++f) out[f] = w[f] + (key == kf[f] ? x.u[f] : 0u);
+            };
+            const uint32_t nlev = __reduce_max_sync(0xffffffffu, x.nlev);   // uniform: the loop below has no divergence
+            step();
+            for (uint32_t l = 1; l < nlev; ++l) {
+#pragma unroll
+                for (uint32_t f = 0; f < ND; ++f) X[row + lane * kStride + f] = out[f];
+                __syncwarp();
+#pragma unroll
+                for (uint32_t f = 0; f < ND; ++f) w[f] = X[row + x.from[f]];
+                row ^= kRow;
+                step();
+            }
+#pragma unroll
+            for (uint32_t f = 0; f < ND; ++f)
+                if ((x.last >> f) & 1u) W32[2 * x.c[f]] = out[f];
+            __syncwarp();
+            const uint32_t k = w0 + lane;
+#pragma unroll
+            for (uint32_t f = 0; f < ND; ++f) S.Wf[f][k] = w[f];
+            S.pick[k] = (uint8_t)(key & 7u);
+            S.over[k] = over != 0;
+        }
     };
 
     auto decide = [&](uint32_t buf, uint32_t m) {
         Stage &S = SB[buf];
+        if (first) {
+            for (uint32_t i = lane; i < d.M; i += 32) bound = max(bound, W[i]);
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) bound = max(bound, shfl_xor_u64(bound, o));
+            first = false;
+        }
+        bound = min(bound, kSmallD) + warp_sum_u64((uint32_t)lane < (m + 31) / 32 ? S.wsum[lane] : 0);
+        if (bound < kSmallD) {
+            decide32(S, m);
+            return;
+        }
         volatile uint64_t *const Wv = W;
         for (uint32_t w0 = 0; w0 < m; w0 += 32) {
             const uint32_t k = w0 + lane;
@@ -1248,7 +1495,7 @@ __global__ void __launch_bounds__(Pipe<choice_d_chunk(ND)>::kThreads) k_choice_d
     };
 
     __syncthreads();
-    choice_pipeline<kChunk>(n, stage, decide, emit);
+    choice_pipeline<kChunk, kChunk>(n, stage, decide, emit);
     unsigned __int128 S1 = 0, S2 = 0;
     uint32_t cnt = 0;
     for (uint32_t i = threadIdx.x, k = 0; i < d.M; i += blockDim.x, ++k) {
