@@ -502,14 +502,23 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads, 1) k_choice(DevS
 // the index as of the start of the batch: a warp per request and 32
 // instances, a lane per instance.  The keys resident on an instance are
 // closed under prefixes (see the routing kernel), so a lane tests block 0
-// and, where that is resident (most instances miss it), finds the run's end
-// by bisection; lanes that probe the same block read the same prefix value.
-// Bound by random 16-byte index reads (one to ten a pair).  4,096 agent
-// prompts x 64 instances, GB300: 822 us with a warp per pair testing 32, then
-// 128 blocks a round; 183 us so.
+// and, where that is resident (most instances miss it), finds the run's end:
+// first whether it is the longer of the runs on the request's two candidates
+// (a shared prefix that is resident on several instances mostly ends at the
+// same block), then by three probes a round, each round leaving a quarter of
+// the range; lanes that probe the same block read the same prefix value.
+// Bound by dependent 16-byte index reads.  4,096 agent prompts x 64
+// instances, GB300: 822 us with a warp per pair testing 32, then 128 blocks a
+// round; 220 us by bisection (ten rounds of one probe); 130 us so.
 constexpr int kAllBlock = 256;
 
-__global__ void __launch_bounds__(kAllBlock) k_probe_all(DevState d, uint32_t n) {
+// resident_at past the home slot (not inlined: three of these in a round).
+static __device__ __noinline__ bool resident_past_home(const Slot *t, uint64_t mask, uint64_t key, uint64_t home,
+                                                       uint64_t front, uint32_t *err, uint64_t loop_limit) {
+    return table_pos1(t, mask, key, home, err, loop_limit) > front;
+}
+
+__global__ void __launch_bounds__(kAllBlock, 4) k_probe_all(DevState d, uint32_t n) {
     pdl_enter();
     if (has_err(d.err)) return;
     const int lane = threadIdx.x & 31;
@@ -525,19 +534,45 @@ __global__ void __launch_bounds__(kAllBlock) k_probe_all(DevState d, uint32_t n)
             const uint64_t *pl = d.plocal + d.r_blkoff[r];
             const Slot *t = d.table[i];
             const uint64_t front = d.log_front[i];
-            auto resident = [&](uint32_t b) {
-                const uint64_t carry = d.seg_carry[s0 + b / kSegBlocks];
-                const uint64_t key = cache_key(pl[b] + carry, d.Sc);
-                const uint64_t anchor = cache_key(pl[b & ~(kGroup - 1)] + carry, d.Sc);
-                const uint64_t home = group_home(anchor, b, mask);
-                return resident_at(t, mask, key, home, front, load_slot(t + home), d.err, d.loop_limit);
+            // which of blocks b[0 .. 2] are resident
+            auto resident = [&](const uint32_t (&b)[3], bool (&in)[3]) {
+                uint64_t key[3], home[3];
+                Slot sl[3];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const uint64_t carry = d.seg_carry[s0 + b[q] / kSegBlocks];
+                    key[q] = cache_key(pl[b[q]] + carry, d.Sc);
+                    home[q] = group_home(cache_key(pl[b[q] & ~(kGroup - 1)] + carry, d.Sc), b[q], mask);
+                    sl[q] = load_slot(t + home[q]);
+                }
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    in[q] = sl[q].key == key[q] ? sl[q].pos1 > front
+                                                : sl[q].key != 0 && resident_past_home(t, mask, key[q], home[q], front,
+                                                                                       d.err, d.loop_limit);
             };
-            if (resident(0)) {
+            const uint64_t key0 = cache_key(pl[0] + d.seg_carry[s0], d.Sc), home0 = group_home(key0, 0, mask);
+            if (resident_at(t, mask, key0, home0, front, load_slot(t + home0), d.err, d.loop_limit)) {
                 uint32_t lo = 0, hi = nblk;   // block lo is resident; hi is not, or the prompt's end
+                const uint32_t g = max(min(d.r_m1[r], nblk), min(d.r_m2[r], nblk));   // first miss on a candidate
+                uint32_t b[3] = {max(g, 1u) - 1, min(g, nblk - 1), nblk / 2};
+                if (g == 0) b[0] = nblk / 4;
+                if (b[2] < b[0]) b[2] = b[0];
                 while (hi - lo > 1) {
-                    const uint32_t mid = lo + (hi - lo) / 2;
-                    if (resident(mid)) lo = mid;
-                    else hi = mid;
+                    bool in[3];
+                    resident(b, in);
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {   // the resident blocks are a leading run: any order of the three
+                        if (in[q]) lo = max(lo, b[q]);
+                        else hi = min(hi, b[q]);
+                    }
+                    const uint32_t step = (hi - lo) / 4, rest = (hi - lo) & 3u;
+                    b[0] = lo + step + (rest > 2);
+                    b[1] = lo + 2 * step + (rest > 1);
+                    b[2] = min(hi - 1, lo + 3 * step + rest);
+                    b[0] = max(b[0], lo + 1);
+                    b[1] = max(b[1], b[0]);
+                    b[2] = max(b[2], b[1]);
                 }
                 h = hi;
             }
