@@ -130,17 +130,19 @@ struct Pipe {
     static constexpr uint32_t kThreads = 32 * (1 + kWorkers + (kWorkers - 1) / 3);
 };
 
-// stage(buffer, k, m, base), decide(buffer, m), emit(buffer, k, m, base): k
+// begin() by the deciding warp while the first chunk is staged; stage(buffer, k,
+// m, base), decide(buffer, m), emit(buffer, k, m, base): k
 // the thread's number among its role's (an emitting thread's request of the
 // chunk; whole windows call, k >= m past the batch's end), m the chunk's
 // requests, base its first request.
-template <uint32_t kChunk, uint32_t kStageThreads, class StageF, class DecideF, class EmitF>
-__device__ __forceinline__ void choice_pipeline(uint32_t n, StageF stage, DecideF decide, EmitF emit) {
+template <uint32_t kChunk, uint32_t kStageThreads, class BeginF, class StageF, class DecideF, class EmitF>
+__device__ __forceinline__ void choice_pipeline(uint32_t n, BeginF begin, StageF stage, DecideF decide, EmitF emit) {
     const uint32_t nc = (n + kChunk - 1) / kChunk, wid = threadIdx.x >> 5;
     const uint32_t w = 32 * (wid - 1 - wid / 4) + (threadIdx.x & 31);   // number among the workers (wid % 4 != 0)
     for (uint32_t t = 0; t < nc + 2; ++t) {
         if (wid == 0) {
-            if (t >= 1 && t <= nc) decide((t - 1) % 3, min(kChunk, n - (t - 1) * kChunk));
+            if (t == 0) begin();
+            else if (t <= nc) decide((t - 1) % 3, min(kChunk, n - (t - 1) * kChunk));
         } else if (wid % 4 == 0) {
         } else if (w < kChunk) {
             if (t >= 2) emit((t - 2) % 3, w, min(kChunk, n - (t - 2) * kChunk), (t - 2) * kChunk);
@@ -165,8 +167,9 @@ __device__ __forceinline__ uint32_t window_links(const uint32_t (&c)[ND], bool v
     uint32_t later = 0;
 #pragma unroll
     for (uint32_t f = 0; f < ND; ++f) from[f] = kNone;
+    const int held = __popc(__ballot_sync(0xffffffffu, valid));   // the valid lanes are the first ones
 #pragma unroll 4
-    for (int j = 0; j < 32; ++j) {
+    for (int j = 0; j < held; ++j) {
         const bool before = j < lane, after = j > lane;
 #pragma unroll
         for (uint32_t y = 0; y < ND; ++y) {
@@ -203,6 +206,8 @@ __device__ __forceinline__ uint32_t window_links(const uint32_t (&c)[ND], bool v
 // the rule compares TTFTs) and tieb set where a tie goes to b (= c1).
 constexpr uint32_t kChoiceChunk = 256;
 constexpr uint64_t kSmall = 1ull << 30;   // loads below it are decided in 32 bits
+constexpr uint32_t kWorkShift = 10;
+constexpr uint64_t kWorkUnit = (1ull << kWorkShift) - 1;
 struct ChoiceStage {
     uint64_t ua[kChoiceChunk], ub[kChoiceChunk];
     int64_t thr[kChoiceChunk];
@@ -212,7 +217,8 @@ struct ChoiceStage {
     // (pair rules: choose b iff W_b - W_a < lead and W_a > thr)
     uint4 rec[kChoiceChunk];
     int2 lim[kChoiceChunk];
-    uint64_t wsum[kChoiceChunk / 32];   // per window: sum of the larger of both works (each kSmall at most)
+    uint4 req[kChoiceChunk];       // the request's length, blocks and hit tokens on c1 and c2
+    uint32_t wsum[kChoiceChunk / 32];   // per window: sum of the larger of both works, in units of 2^kWorkShift (rounded up)
     uint32_t nlev[kChoiceChunk / 32];
     uint8_t lev[kChoiceChunk], pickb[kChoiceChunk];
 };
@@ -265,6 +271,7 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads, 1) k_choice(DevS
             const uint32_t h1 = hit_tokens(d.r_m1[r], nblk, d.B), h2 = hit_tokens(d.r_m2[r], nblk, d.B);
             const uint32_t c1 = d.r_c1[r], c2 = d.r_c2[r];
             // global cache affinity always takes c1: orient it as a, never b
+            S.req[k] = make_uint4(L, nblk, h1, h2);
             const bool a2 = rule != DM_RULE_CACHE_AFFINITY && h2 > h1;
             const bool differ = h1 != h2;
             const uint64_t ua = cost * (L - (a2 ? h2 : h1)), ub = cost * (L - (a2 ? h1 : h2));
@@ -306,10 +313,10 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads, 1) k_choice(DevS
         }
         S.rec[k] = make_uint4(valid ? ids[0] | ids[1] << 16 : 0, link, u32[0], u32[1]);
         S.lev[k] = valid ? (uint8_t)lev : kNoLevel;
-        most = warp_sum_u64(most);
+        const uint32_t sum = __reduce_add_sync(0xffffffffu, (uint32_t)((most + kWorkUnit) >> kWorkShift));
         if (lane == 0) {
             S.nlev[k / 32] = nlev;
-            S.wsum[k / 32] = most;
+            S.wsum[k / 32] = sum;
         }
     };
 
@@ -320,8 +327,11 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads, 1) k_choice(DevS
     // or branches.  A level is four shuffles and a dozen operations in
     // registers.  The window's last request on an instance leaves its load in
     // W; the next window's staged values are read meanwhile.
-    uint64_t bound = 0;   // no load exceeds it
-    bool first = true;
+    uint64_t bound = 0;   // no load exceeds it, unless it is kSmall
+    auto begin = [&] {
+        for (uint32_t i = lane; i < d.M; i += 32) bound = max(bound, min(d.W[i], kSmall));
+        bound = __reduce_max_sync(0xffffffffu, (uint32_t)bound);
+    };
     auto decide32 = [&](ChoiceStage &S, uint32_t m) {
         volatile uint32_t *const W32 = reinterpret_cast<volatile uint32_t *>(W);   // low words; the high ones are 0
         uint4 nr = S.rec[lane];
@@ -373,13 +383,9 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads, 1) k_choice(DevS
 
     auto decide = [&](uint32_t buf, uint32_t m) {
         ChoiceStage &S = SB[buf];
-        if (first) {
-            for (uint32_t i = lane; i < d.M; i += 32) bound = max(bound, W[i]);
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) bound = max(bound, shfl_xor_u64(bound, o));
-            first = false;
-        }
-        bound = min(bound, kSmall) + warp_sum_u64((uint32_t)lane < (m + 31) / 32 ? S.wsum[lane] : 0);
+        bound = min(bound + (uint64_t(__reduce_add_sync(0xffffffffu, (uint32_t)lane < (m + 31) / 32 ? S.wsum[lane] : 0))
+                             << kWorkShift),
+                    kSmall);
         if (bound < kSmall) {
             decide32(S, m);
             return;
@@ -429,7 +435,9 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads, 1) k_choice(DevS
         const bool a_is_c2 = (ab >> 28) & 1, differ = (ab >> 29) & 1;
         const bool pb = valid && S.pickb[k];
         const uint32_t ch = pb ? b : a;
-        const uint32_t nbr = valid ? d.r_nblk[r] : 0;
+        const uint4 rq = valid ? S.req[k] : make_uint4(0, 0, 0, 0);
+        const uint32_t L = rq.x, nbr = rq.y, h1 = rq.z, h2 = rq.w;
+        const uint32_t qh = d.q_head[ch];   // (a = 0 past the batch's end)
         const uint64_t pt = record_place<kChoiceChunk>(PT, ch, (uint64_t(nbr) << 32) + 1, valid, k / 32,
                                                        (m + 31) / 32, lane);
         if (!valid) return;
@@ -440,8 +448,6 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads, 1) k_choice(DevS
         o.chosen[r] = ch;
         o.switched[r] = sw;
         d.r_final[r] = ch;
-        const uint32_t L = d.r_L[r];
-        const uint32_t h1 = hit_tokens(d.r_m1[r], nbr, d.B), h2 = hit_tokens(d.r_m2[r], nbr, d.B);
         ms.tokens += L;
         ms.hits += (ch == (a_is_c2 ? b : a)) ? h1 : h2;
         ms.sw += sw;
@@ -449,7 +455,7 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads, 1) k_choice(DevS
         if (ta > slo && tb > slo) d.info->both_over = 1;
         d.r_touchoff[r] = pt >> 32;          // offset among this batch's records of ch
         const uint32_t slot = (uint32_t)pt;
-        if (slot - d.q_head[ch] >= d.Q) {
+        if (slot - qh >= d.Q) {
             set_err(d.err, DM_ERR_CAPACITY);
             return;
         }
@@ -472,8 +478,8 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads, 1) k_choice(DevS
         d.q[uint64_t(ch) * d.Q + (slot & (d.Q - 1))] = e;
     };
 
-    __syncthreads();
-    choice_pipeline<kChoiceChunk, kChoiceChunk>(n, stage, decide, emit);
+    // (W and PT are first read after the first chunk's barrier)
+    choice_pipeline<kChoiceChunk, kChoiceChunk>(n, begin, stage, decide, emit);
     unsigned __int128 S1 = 0, S2 = 0;
     uint32_t cnt = 0;
     for (uint32_t i = threadIdx.x, k = 0; i < d.M; i += blockDim.x, ++k) {
@@ -868,7 +874,7 @@ __global__ void __launch_bounds__(GlobalPipe<J>::kThreads, 1) k_choice_all(DevSt
         d.q[uint64_t(ch) * d.Q + (slot & (d.Q - 1))] = e;
     };
 
-    choice_pipeline<kChunk, kGlobalStageThreads>(n, stage, decide, emit);
+    choice_pipeline<kChunk, kGlobalStageThreads>(n, [] {}, stage, decide, emit);
     unsigned __int128 S1 = 0, S2 = 0;
     uint32_t cnt = 0;
     for (uint32_t i = threadIdx.x; i < d.M; i += blockDim.x) {
@@ -1233,7 +1239,7 @@ struct ChoiceStageD {
     uint16_t c[ND][kChunk];
     uint8_t most[kChunk];             // bit f: candidate f has the most hit tokens
     uint8_t lev[kChunk], pick[kChunk], over[kChunk];
-    uint64_t wsum[kChunk / 32];       // per window: sum of the largest works (each kSmallD at most)
+    uint32_t wsum[kChunk / 32];       // per window: sum of the largest works, in units of 2^kWorkShift (rounded up)
     uint32_t u32[ND][kChunk];         // low words of u
     uint16_t from[ND][kChunk];        // word of the exchange rows that holds candidate f's load
     uint8_t last[kChunk];             // bit f: no later request of the window names candidate f
@@ -1313,10 +1319,10 @@ __global__ void __launch_bounds__(Pipe<choice_d_chunk(ND)>::kThreads, 1) k_choic
             S.c[f][k] = valid ? (uint16_t)ids[f] : 0;   // every lane of a window reads its loads
             S.from[f][k] = (uint16_t)(valid && from[f] != kNone ? from[f] : (32 + lane) * kStride + f);
         }
-        umax = warp_sum_u64(min(umax, kSmallD));
+        const uint32_t sum = __reduce_add_sync(0xffffffffu, (uint32_t)((min(umax, kSmallD) + kWorkUnit) >> kWorkShift));
         if (lane == 0) {
             S.nlev[k / 32] = nlev;
-            S.wsum[k / 32] = umax;
+            S.wsum[k / 32] = sum;
         }
     };
 
@@ -1326,8 +1332,7 @@ __global__ void __launch_bounds__(Pipe<choice_d_chunk(ND)>::kThreads, 1) k_choic
     // number, so one minimum over the candidates gives the least loaded and
     // the earlier ring on ties; the candidates with the most hit tokens have
     // the same uncached work.
-    uint64_t bound = 0;   // no load exceeds it
-    bool first = true;
+    uint64_t bound = 0;   // no load exceeds it, unless it is kSmallD
     struct Win {
         uint32_t nlev, most, last, c[ND], u[ND], from[ND];
     };
@@ -1344,6 +1349,10 @@ __global__ void __launch_bounds__(Pipe<choice_d_chunk(ND)>::kThreads, 1) k_choic
             x.from[f] = S.from[f][k];
         }
         return x;
+    };
+    auto begin = [&] {
+        for (uint32_t i = lane; i < d.M; i += 32) bound = max(bound, min(d.W[i], kSmallD));
+        bound = __reduce_max_sync(0xffffffffu, (uint32_t)bound);
     };
     auto decide32 = [&](Stage &S, uint32_t m) {
         volatile uint32_t *const W32 = reinterpret_cast<volatile uint32_t *>(W);   // low words; the high ones are 0
@@ -1417,13 +1426,9 @@ __global__ void __launch_bounds__(Pipe<choice_d_chunk(ND)>::kThreads, 1) k_choic
 
     auto decide = [&](uint32_t buf, uint32_t m) {
         Stage &S = SB[buf];
-        if (first) {
-            for (uint32_t i = lane; i < d.M; i += 32) bound = max(bound, W[i]);
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) bound = max(bound, shfl_xor_u64(bound, o));
-            first = false;
-        }
-        bound = min(bound, kSmallD) + warp_sum_u64((uint32_t)lane < (m + 31) / 32 ? S.wsum[lane] : 0);
+        bound = min(bound + (uint64_t(__reduce_add_sync(0xffffffffu, (uint32_t)lane < (m + 31) / 32 ? S.wsum[lane] : 0))
+                             << kWorkShift),
+                    kSmallD);
         if (bound < kSmallD) {
             decide32(S, m);
             return;
@@ -1487,7 +1492,7 @@ __global__ void __launch_bounds__(Pipe<choice_d_chunk(ND)>::kThreads, 1) k_choic
         const bool valid = k < m;
         const uint32_t r = base + k, pick = valid ? S.pick[k] : 0;
         const uint32_t ch = valid ? S.c[pick][k] : 0;
-        const uint32_t nbr = valid ? d.r_nblk[r] : 0;
+        const uint32_t nbr = valid ? d.r_nblk[r] : 0, L = valid ? d.r_L[r] : 0, qh = d.q_head[ch];
         const uint64_t pt = record_place<kChunk>(PT, ch, (uint64_t(nbr) << 32) + 1, valid, k / 32, (m + 31) / 32,
                                                  lane);
         if (!valid) return;
@@ -1503,14 +1508,13 @@ __global__ void __launch_bounds__(Pipe<choice_d_chunk(ND)>::kThreads, 1) k_choic
         o.switched[r] = S.over[k];
         d.r_final[r] = ch;
         d.r_touchoff[r] = pt >> 32;   // offset among this batch's records of ch
-        const uint32_t L = d.r_L[r];
         const uint32_t *h = d.rd_hit + uint64_t(r) * ND;
         ms.tokens += L;
         ms.hits += h[pick];
         ms.sw += S.over[k];
         ms.est += S.Wf[pick][k] + S.u[pick][k] <= slo;
         const uint32_t slot = (uint32_t)pt;
-        if (slot - d.q_head[ch] >= d.Q) {
+        if (slot - qh >= d.Q) {
             set_err(d.err, DM_ERR_CAPACITY);
             return;
         }
@@ -1529,8 +1533,8 @@ __global__ void __launch_bounds__(Pipe<choice_d_chunk(ND)>::kThreads, 1) k_choic
         d.q[uint64_t(ch) * d.Q + (slot & (d.Q - 1))] = e;
     };
 
-    __syncthreads();
-    choice_pipeline<kChunk, kChunk>(n, stage, decide, emit);
+    // (W and PT are first read after the first chunk's barrier)
+    choice_pipeline<kChunk, kChunk>(n, begin, stage, decide, emit);
     unsigned __int128 S1 = 0, S2 = 0;
     uint32_t cnt = 0;
     for (uint32_t i = threadIdx.x, k = 0; i < d.M; i += blockDim.x, ++k) {
