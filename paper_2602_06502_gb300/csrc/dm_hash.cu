@@ -344,31 +344,25 @@ __device__ __forceinline__ void probe_segment(const uint64_t (&key)[2], uint32_t
                                               uint64_t lim, int lane, uint32_t &m1, uint32_t &m2) {
     uint64_t home[2];
     Slot s1[2], s2[2];
+    int look[2][2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const uint32_t b = base + 32 * k + lane;
         home[k] = group_home(group_anchor(key[k], lane), b, mask);
-        const bool inb = b < end;
-        s1[k] = (inb && do1) ? load_slot(rv.t1 + home[k]) : Slot{0, 0};
-        s2[k] = (inb && do2) ? load_slot(rv.t2 + home[k]) : Slot{0, 0};
+        s1[k] = (b < end && do1) ? load_slot(rv.t1 + home[k]) : Slot{0, 0};   // (an empty slot: missing)
+        s2[k] = (b < end && do2) ? load_slot(rv.t2 + home[k]) : Slot{0, 0};
     }
-    m1 = kNoMiss;
-    m2 = kNoMiss;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-        const uint32_t b = base + 32 * k + lane;
-        const bool inb = b < end;
-        if (do1) {
-            const bool miss = inb && !resident_at(rv.t1, mask, key[k], home[k], rv.f1, s1[k], err, lim);
-            const uint32_t bal = __ballot_sync(0xffffffffu, miss);
-            if (bal && m1 == kNoMiss) m1 = base + 32 * k + __ffs(bal) - 1;
-        }
-        if (do2) {
-            const bool miss = inb && !resident_at(rv.t2, mask, key[k], home[k], rv.f2, s2[k], err, lim);
-            const uint32_t bal = __ballot_sync(0xffffffffu, miss);
-            if (bal && m2 == kNoMiss) m2 = base + 32 * k + __ffs(bal) - 1;
-        }
+        look[0][k] = look_at(s1[k], key[k], rv.f1);
+        look[1][k] = look_at(s2[k], key[k], rv.f2);
     }
+    const Slot *const t[2] = {rv.t1, rv.t2};
+    const uint64_t front[2] = {rv.f1, rv.f2};
+    uint32_t first[2];
+    leading_runs<2, 2>(look, t, front, mask, key, home, lane, err, lim, first);
+    m1 = do1 && base + first[0] < end ? base + first[0] : kNoMiss;
+    m2 = do2 && base + first[1] < end ? base + first[1] : kNoMiss;
 }
 
 // Cache keys of head segment s of request r (nb blocks, f1 carry `carry`
@@ -448,19 +442,21 @@ __device__ __noinline__ void tail_task(const DevState &d, uint32_t r, int lane) 
             if (!(f ? open2 : open1)) continue;
             const Slot *t = f ? rv.t2 : rv.t1;
             const uint64_t front = f ? rv.f2 : rv.f1;
+            uint64_t home[kTailVec];
             Slot sl[kTailVec];
-#pragma unroll
-            for (uint32_t q = 0; q < kTailVec; ++q)
-                sl[q] = j0 + 32 * q + lane < nseg ? load_slot(t + group_home(key[q], 0, mask)) : Slot{0, 0};
-            uint32_t jf = end;
+            int look[1][kTailVec];
 #pragma unroll
             for (uint32_t q = 0; q < kTailVec; ++q) {
-                const uint32_t sg = j0 + 32 * q + lane;
-                const bool miss = sg < nseg && !resident_at(t, mask, key[q], group_home(key[q], 0, mask), front,
-                                                            sl[q], d.err, d.loop_limit);
-                const uint32_t bal = __ballot_sync(0xffffffffu, miss);
-                if (bal && jf == end) jf = j0 + 32 * q + __ffs(bal) - 1;
+                home[q] = group_home(key[q], 0, mask);
+                sl[q] = j0 + 32 * q + lane < nseg ? load_slot(t + home[q]) : Slot{0, 0};
             }
+#pragma unroll
+            for (uint32_t q = 0; q < kTailVec; ++q) look[0][q] = look_at(sl[q], key[q], front);   // past the end: missing
+            const Slot *const tf[1] = {t};
+            const uint64_t ff[1] = {front};
+            uint32_t run[1];
+            leading_runs<1, (int)kTailVec>(look, tf, ff, mask, key, home, lane, d.err, d.loop_limit, run);
+            const uint32_t jf = min(end, j0 + run[0]);
             if (jf == end && end < nseg) continue;   // goes on in the next round
             // the run ends in segment jf - 1 or at block 64 jf (past the
             // last segment: the whole prompt); the head is resident
@@ -545,19 +541,23 @@ __device__ __noinline__ bool route_task(const DevState &d, const uint32_t *token
     rv.f1 = d.log_front[a];   // resident: record at or after the front (as of the batch's start)
     rv.f2 = d.log_front[b];
     const uint64_t mask = d.S - 1;
-    // first block of every head segment on both candidates (lane s: segment s)
-    bool miss1 = true, miss2 = true;
+    // first block of every head segment on both candidates (lane s: segment
+    // s).  j_f: the first head segment whose first block is missing on c_f
+    // (hs: none; lanes >= hs count as missing, and a head of 32 segments has
+    // no such lane)
+    const uint64_t key0[1] = {cache_key(carry + pf, d.Sc)};
+    const uint64_t home0[1] = {group_home(key0[0], 0, mask)};   // a segment's first block anchors its own group
+    int look[2][1] = {{kOut}, {kOut}};
     if ((uint32_t)lane < hs) {
-        const uint64_t key = cache_key(carry + pf, d.Sc);
-        const uint64_t home = group_home(key, 0, mask);   // a segment's first block anchors its own group
-        miss1 = !resident_at(rv.t1, mask, key, home, rv.f1, load_slot(rv.t1 + home), d.err, d.loop_limit);
-        miss2 = !resident_at(rv.t2, mask, key, home, rv.f2, load_slot(rv.t2 + home), d.err, d.loop_limit);
+        const Slot a1 = load_slot(rv.t1 + home0[0]), a2 = load_slot(rv.t2 + home0[0]);
+        look[0][0] = look_at(a1, key0[0], rv.f1);
+        look[1][0] = look_at(a2, key0[0], rv.f2);
     }
-    // j_f: the first head segment whose first block is missing on c_f (hs:
-    // none; lanes >= hs count as missing, and a head of 32 segments has no
-    // such lane)
-    const uint32_t b1 = __ballot_sync(0xffffffffu, miss1), b2 = __ballot_sync(0xffffffffu, miss2);
-    const uint32_t j1 = b1 ? __ffs(b1) - 1 : 32u, j2 = b2 ? __ffs(b2) - 1 : 32u;
+    const Slot *const tabs[2] = {rv.t1, rv.t2};
+    const uint64_t fronts[2] = {rv.f1, rv.f2};
+    uint32_t run[2];
+    leading_runs<2, 1>(look, tabs, fronts, mask, key0, home0, lane, d.err, d.loop_limit, run);
+    const uint32_t j1 = run[0], j2 = run[1];
     // the run on c_f ends in segment j_f - 1 or at block 64 j_f (when j_f <
     // hs); probe that segment, once for both candidates when they agree
     uint32_t m1 = j1 == 0 ? 0 : kNoMiss, m2 = j2 == 0 ? 0 : kNoMiss;

@@ -754,6 +754,156 @@ __device__ __forceinline__ bool resident_at(const Slot *t, uint64_t mask, uint64
     return table_pos1(t, mask, key, home, err, loop_limit) > front;
 }
 
+// Leading runs.  The keys resident on an instance are closed under prefixes (a
+// request touches its keys from its last block down into an exact LRU), so of
+// a prompt's blocks a leading run is resident, and a lookup that its home slot
+// leaves open (the slot holds another key) matters only between the last block
+// known resident and the first known missing.  Those are settled from the
+// lowest up, eight lanes to a lookup and a slot to a lane: the first three
+// buckets of eight lookups (four on each of two instances) in one round trip
+// of six coalesced loads.  The first or second of them mostly is the run's
+// end.  Every lane walking its own open lookups read a bucket by eight loads of
+// its own: 2.5 to 3.5 us a walk of one or two round trips.
+enum Look : int { kOut, kIn, kOpen };   // missing, resident, not known from the slots seen
+
+__device__ __forceinline__ int look_at(const Slot &s, uint64_t key, uint64_t front) {
+    return s.key == key ? (s.pos1 > front ? kIn : kOut) : s.key == 0 ? kOut : kOpen;
+}
+
+// What a bucket (a slot in each of the group's eight lanes) says of the
+// group's key: found there, or room there (an insert takes the first empty slot
+// of its probe order, and slots never empty), or open.  Whole warp.
+__device__ __forceinline__ int look_bucket(const Slot &s, uint64_t key, uint64_t front, int gbase) {
+    const uint32_t m = (__ballot_sync(0xffffffffu, s.key == key) >> gbase) & 0xFFu;
+    const uint32_t e = (__ballot_sync(0xffffffffu, s.key == 0) >> gbase) & 0xFFu;
+    const uint64_t p = shfl_u64(s.pos1, gbase + (m ? __ffs(m) - 1 : 0));
+    return m ? (p > front ? kIn : kOut) : e ? kOut : kOpen;
+}
+
+// Leading resident blocks on F instances (one or two: tables t, log fronts
+// front) among blocks 32 q + lane (q < K) with these keys and homes; st: what
+// the home slots say, blocks past the end kOut.  first[f]: the first missing
+// block on instance f (32 K: none).  Whole warp.
+template <int F, int K>
+__device__ __forceinline__ void leading_runs(const int (&st)[F][K], const Slot *const (&t)[F], const uint64_t (&front)[F],
+                                             uint64_t mask, const uint64_t (&key)[K], const uint64_t (&home)[K],
+                                             int lane, uint32_t *err, uint64_t loop_limit, uint32_t (&first)[F]) {
+    static_assert(kGroup == 8 && (F == 1 || F == 2), "eight lanes to a bucket");
+    uint32_t u[F][K], any = 0;   // open lanes that matter
+#pragma unroll
+    for (int f = 0; f < F; ++f) {
+        int last = -1;
+        first[f] = 32 * K;
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+            const uint32_t out = __ballot_sync(0xffffffffu, st[f][q] == kOut);
+            const uint32_t in = __ballot_sync(0xffffffffu, st[f][q] == kIn);
+            u[f][q] = ~(out | in);
+            if (out && first[f] == 32 * K) first[f] = 32 * q + __ffs(out) - 1;
+            if (in) last = 32 * q + 31 - __clz(in);
+        }
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+            const int lo = last + 1 - 32 * q, hi = (int)first[f] - 32 * q;   // lanes lo .. hi - 1 of the word
+            const uint32_t below = hi >= 32 ? ~0u : hi <= 0 ? 0u : (1u << hi) - 1u;
+            const uint32_t under = lo >= 32 ? ~0u : lo <= 0 ? 0u : (1u << lo) - 1u;
+            u[f][q] &= below & ~under;
+            any |= u[f][q];
+        }
+    }
+    constexpr uint32_t kPer = F == 2 ? 4 : 8;   // lookups of an instance in a round
+    const int g = lane >> 3, gbase = lane & 24;
+    while (any) {
+        // the round's lookups: group g takes the g-th lowest open block of
+        // each instance, or the g-th and the (g + 4)-th of the only one, all
+        // of an instance in its first word with open ones
+        int q[F], b[2];
+        uint32_t w[F];
+        bool has[2];
+        uint64_t k[2], R0[2];
+        Slot s0[2], s1[2], s2[2];
+#pragma unroll
+        for (int f = 0; f < F; ++f) {
+            q[f] = 0;
+            w[f] = u[f][0];
+#pragma unroll
+            for (int x = 1; x < K; ++x)
+                if (!w[f]) {
+                    w[f] = u[f][x];
+                    q[f] = x;
+                }
+        }
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            const int f = F == 2 ? x : 0;
+            uint32_t o = w[f];
+#pragma unroll
+            for (int i = 0; i < (int)kPer - 1; ++i)
+                if (i < (F == 2 ? g : g + 4 * x)) o &= o - 1;
+            has[x] = o != 0;
+            b[x] = has[x] ? __ffs(o) - 1 : 0;
+            uint64_t kq = key[0], hq = home[0];
+#pragma unroll
+            for (int y = 1; y < K; ++y)
+                if (q[f] == y) {
+                    kq = key[y];
+                    hq = home[y];
+                }
+            k[x] = shfl_u64(kq, b[x]);
+            R0[x] = shfl_u64(hq, b[x]) & ~uint64_t(kGroup - 1);
+            const Slot *p = t[f] + (lane & 7);
+            s0[x] = has[x] ? load_slot(p + R0[x]) : Slot{0, 0};
+            s1[x] = has[x] ? load_slot(p + probe_bucket(1, R0[x], k[x], mask)) : Slot{0, 0};
+            s2[x] = has[x] ? load_slot(p + probe_bucket(2, R0[x], k[x], mask)) : Slot{0, 0};
+        }
+        uint32_t outs[2];   // lanes of the groups whose lookup is missing
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            const int f = F == 2 ? x : 0;
+            const uint64_t fr = front[f];
+            int r = look_bucket(s0[x], k[x], fr, gbase);
+            const int r1 = look_bucket(s1[x], k[x], fr, gbase), r2 = look_bucket(s2[x], k[x], fr, gbase);
+            r = r != kOpen ? r : r1 != kOpen ? r1 : r2;
+            const uint64_t walk = (mask >> 3) + kLinearBuckets + 1;
+            for (uint64_t j = 3; __any_sync(0xffffffffu, r == kOpen); ++j) {   // (no lookup: found room)
+                const bool open = r == kOpen;
+                Slot sj{0, 0};
+                if (open) sj = load_slot(t[f] + probe_bucket(j, R0[x], k[x], mask) + (lane & 7));
+                const int rj = look_bucket(sj, k[x], fr, gbase);
+                if (open) r = rj;
+                if (j > walk || (loop_limit && j > loop_limit)) {
+                    if (r == kOpen) {
+                        set_err(err, DM_ERR_TIMEOUT);
+                        r = kOut;
+                    }
+                }
+            }
+            outs[x] = __ballot_sync(0xffffffffu, has[x] && r == kOut);
+        }
+        any = 0;
+#pragma unroll
+        for (int f = 0; f < F; ++f) {
+            // the lowest missing one ends the run; else the round's are resident
+            uint32_t end = 32;
+#pragma unroll
+            for (int x = F == 2 ? f : 1; x >= (F == 2 ? f : 0); --x) {
+                const int bb = __shfl_sync(0xffffffffu, b[x], outs[x] ? __ffs(outs[x]) - 1 : 0);
+                if (outs[x]) end = bb;
+            }
+            if (end < 32) first[f] = min(first[f], 32u * q[f] + end);
+            uint32_t rest = w[f];
+#pragma unroll
+            for (int i = 0; i < (int)kPer; ++i) rest &= rest - 1;
+#pragma unroll
+            for (int x = 0; x < K; ++x) {
+                if (x == q[f]) u[f][x] = rest;
+                if (end < 32) u[f][x] = 0;
+                any |= u[f][x];
+            }
+        }
+    }
+}
+
 // Adaptive hash-prefix length (Sec. 3.2): the walk from min(K_route, n_blk)
 // blocks, one step deeper while the node (the key of the prefix's last
 // block) is expanded.  Level j sits at depth min(d0 + j * step, cap), so
