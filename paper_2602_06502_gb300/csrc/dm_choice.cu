@@ -1138,7 +1138,8 @@ cudaError_t launch_choice(const DevState &d, const dm_route_out &o, uint32_t n, 
 //               (function 1 from the prefix values; functions 2..d hash the
 //               first K blocks here), a successor search on each ring, the
 //               distinct fix, and the leading run of resident blocks on
-//               each candidate;
+//               each candidate (4,096 agent prompts, d = 4: 72 us when it
+//               walked 32 blocks a round, 50 us by segments);
 //   k_choice_d  one CTA: DualMap's SLO-aware rule over d candidates in
 //               arrival order (the choice pipeline), queue appends, the
 //               commit's per-request offsets and the batch's metrics,
@@ -1205,27 +1206,74 @@ __global__ void k_route_d(DevState d, const uint32_t *tokens, uint32_t n) {
         }
         cand[f] = x;
     }
-    // leading run of resident blocks on each candidate (index as of the start of the batch)
+    // leading run of resident blocks on each candidate (index as of the start
+    // of the batch), two candidates at a time: the first block of every
+    // segment, 32 segments a round, then the segment that holds the run's end
     const uint64_t mask = d.S - 1;
-    for (uint32_t f = 0; f < nd; ++f) {
-        const Slot *t = d.table[cand[f]];
-        const uint64_t front = d.log_front[cand[f]];
-        uint32_t h = nblk;
-        for (uint32_t base = 0; base < nblk; base += 32) {
-            const uint32_t b = base + lane;
-            const bool inb = b < nblk;
-            const uint64_t key = inb ? cache_key(d.plocal[bo + b] + d.seg_carry[s0 + b / kSegBlocks], d.Sc) : 0;
-            const uint64_t home = group_home(group_anchor(key, lane), b, mask);
-            const bool miss = inb && !resident_at(t, mask, key, home, front, load_slot(t + home), d.err, d.loop_limit);
-            const uint32_t bal = __ballot_sync(0xffffffffu, miss);
-            if (bal) {
-                h = base + __ffs(bal) - 1;
-                break;
+    const uint32_t nseg = (nblk + kSegBlocks - 1) / kSegBlocks;
+    for (uint32_t f0 = 0; f0 < nd; f0 += 2) {
+        const bool two = f0 + 1 < nd;
+        const uint32_t ca = cand[f0], cb = two ? cand[f0 + 1] : ca;
+        const Slot *const t[2] = {d.table[ca], d.table[cb]};
+        const uint64_t front[2] = {d.log_front[ca], d.log_front[cb]};
+        uint32_t js[2] = {nseg, two ? nseg : 0}, m[2];   // first segment whose first block is missing
+        bool open[2] = {true, two};
+        for (uint32_t g0 = 0; g0 < nseg && (open[0] || open[1]); g0 += 32) {
+            const uint32_t sg = g0 + lane;
+            const uint64_t key[1] = {
+                sg < nseg ? cache_key(d.plocal[bo + uint64_t(sg) * kSegBlocks] + d.seg_carry[s0 + sg], d.Sc) : 0};
+            const uint64_t home[1] = {group_home(key[0], 0, mask)};   // a segment's first block anchors its own group
+            Slot s[2];
+            int look[2][1];
+#pragma unroll
+            for (int x = 0; x < 2; ++x) s[x] = sg < nseg && open[x] ? load_slot(t[x] + home[0]) : Slot{0, 0};
+#pragma unroll
+            for (int x = 0; x < 2; ++x) look[x][0] = sg < nseg ? look_at(s[x], key[0], front[x]) : kOut;
+            uint32_t run[2];
+            leading_runs<2, 1>(look, t, front, mask, key, home, lane, d.err, d.loop_limit, run);
+#pragma unroll
+            for (int x = 0; x < 2; ++x)
+                if (open[x] && run[x] < min(32u, nseg - g0)) {
+                    js[x] = g0 + run[x];
+                    open[x] = false;
+                }
+        }
+#pragma unroll
+        for (int x = 0; x < 2; ++x) m[x] = min(js[x] * kSegBlocks, nblk);
+#pragma unroll 1
+        for (int x = 0; x < 2; ++x) {
+            if (js[x] == 0 || (x == 1 && js[1] == js[0])) continue;
+            const uint32_t c0 = (js[x] - 1) * kSegBlocks, cn = min(kSegBlocks, nblk - c0);
+            const uint64_t carry = d.seg_carry[s0 + js[x] - 1];
+            uint64_t key[2], home[2];
+            Slot s[2][2];
+            int look[2][2];
+            const bool in[2] = {x == 0, js[1] == js[x]};
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const uint32_t e = 32 * q + lane;
+                key[q] = e < cn ? cache_key(d.plocal[bo + c0 + e] + carry, d.Sc) : 0;
+                home[q] = group_home(group_anchor(key[q], lane), c0 + e, mask);
+#pragma unroll
+                for (int y = 0; y < 2; ++y) s[y][q] = e < cn && in[y] ? load_slot(t[y] + home[q]) : Slot{0, 0};
             }
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+                for (int y = 0; y < 2; ++y) look[y][q] = 32u * q + lane < cn ? look_at(s[y][q], key[q], front[y]) : kOut;
+            uint32_t run[2];
+            leading_runs<2, 2>(look, t, front, mask, key, home, lane, d.err, d.loop_limit, run);
+#pragma unroll
+            for (int y = 0; y < 2; ++y)
+                if (in[y] && run[y] < cn) m[y] = c0 + run[y];
         }
         if (lane == 0) {
-            d.rd_cand[uint64_t(r) * nd + f] = cand[f];
-            d.rd_hit[uint64_t(r) * nd + f] = h * B;
+            d.rd_cand[uint64_t(r) * nd + f0] = ca;
+            d.rd_hit[uint64_t(r) * nd + f0] = m[0] * B;
+            if (two) {
+                d.rd_cand[uint64_t(r) * nd + f0 + 1] = cb;
+                d.rd_hit[uint64_t(r) * nd + f0 + 1] = m[1] * B;
+            }
         }
     }
     if (lane == 0) d.r_K[r] = K;

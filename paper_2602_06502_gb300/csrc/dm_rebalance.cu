@@ -96,34 +96,37 @@ static __device__ __noinline__ uint32_t ring_leading_run(const DevState &d, cons
     const uint64_t front = d.log_front[j], mask = d.S - 1, km = d.KQ - 1;
     const uint32_t nseg = (nblk + kSegBlocks - 1) / kSegBlocks;
     uint32_t js = nseg;   // first segment whose first block is missing (nseg: none)
+    const Slot *const ts[1] = {t};
+    const uint64_t fronts[1] = {front};
+    uint32_t run[1];
     for (uint32_t s0 = 0; s0 < nseg; s0 += 32) {
         const uint32_t sg = s0 + lane;
-        bool miss = false;
-        if (sg < nseg) {
-            const uint64_t key = ring[(koff + uint64_t(sg) * kSegBlocks) & km];
-            const uint64_t home = group_home(key, 0, mask);   // a segment's first block anchors its own group
-            miss = !resident_at(t, mask, key, home, front, load_slot(t + home), d.err, d.loop_limit);
-        }
-        const uint32_t bal = __ballot_sync(0xffffffffu, miss);
-        if (bal) {
-            js = s0 + __ffs(bal) - 1;
+        const uint64_t key[1] = {sg < nseg ? ring[(koff + uint64_t(sg) * kSegBlocks) & km] : 0};
+        const uint64_t home[1] = {group_home(key[0], 0, mask)};   // a segment's first block anchors its own group
+        const int look[1][1] = {{sg < nseg ? look_at(load_slot(t + home[0]), key[0], front) : kOut}};
+        leading_runs<1, 1>(look, ts, fronts, mask, key, home, lane, d.err, d.loop_limit, run);
+        if (run[0] < min(32u, nseg - s0)) {
+            js = s0 + run[0];
             break;
         }
     }
     if (js == 0) return 0;
     // the run ends in segment js - 1, or at block 64 js
     const uint32_t c0 = (js - 1) * kSegBlocks, cn = min(kSegBlocks, nblk - c0);
-    uint32_t first = 0xFFFFFFFFu;
+    uint64_t key[2], home[2];
+    Slot s[2];
+    int look[1][2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const uint32_t b = 32 * k + lane;
-        const uint64_t key = b < cn ? ring[(koff + c0 + b) & km] : 0;
-        const uint64_t home = group_home(group_anchor(key, lane), c0 + b, mask);
-        const bool miss = b < cn && !resident_at(t, mask, key, home, front, load_slot(t + home), d.err, d.loop_limit);
-        const uint32_t bal = __ballot_sync(0xffffffffu, miss);
-        if (bal && first == 0xFFFFFFFFu) first = c0 + 32 * k + __ffs(bal) - 1;
+        key[k] = b < cn ? ring[(koff + c0 + b) & km] : 0;
+        home[k] = group_home(group_anchor(key[k], lane), c0 + b, mask);
+        s[k] = b < cn ? load_slot(t + home[k]) : Slot{0, 0};
     }
-    if (first != 0xFFFFFFFFu) return first;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) look[0][k] = 32u * k + lane < cn ? look_at(s[k], key[k], front) : kOut;
+    leading_runs<1, 2>(look, ts, fronts, mask, key, home, lane, d.err, d.loop_limit, run);
+    if (run[0] < cn) return c0 + run[0];
     return js < nseg ? js * kSegBlocks : nblk;
 }
 
