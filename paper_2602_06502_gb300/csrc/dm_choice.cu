@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads, 1) k_choice(DevS
 // the range; lanes that probe the same block read the same prefix value.
 // Bound by dependent 16-byte index reads.  4,096 agent prompts x 64
 // instances, GB300: 822 us with a warp per pair testing 32, then 128 blocks a
-// round; 220 us by bisection (ten rounds of one probe); 130 us so.
+// round; 220 us by bisection (ten rounds of one probe); 90 us so.
 constexpr int kAllBlock = 256;
 
 // resident_at past the home slot (not inlined: three of these in a round).
@@ -603,7 +603,9 @@ __global__ void __launch_bounds__(kAllBlock, 4) k_probe_all(DevState d, uint32_t
 // 4,096 agent prompts on 64 instances, min TTFT, GB300: 1,678 us with 64-bit
 // keys and loads in shared memory, three reductions a request, and staging
 // and emission between the chunks; 922 us when the deciding warp also read
-// and wrote the loads in shared memory for every request; 302 us so.
+// and wrote the loads in shared memory for every request; 302 us with a vote
+// for the winning lane and sums over whole chunks in the emitting warps; 205 us
+// so.
 constexpr uint32_t kGlobalStageThreads = 256;
 template <uint32_t J>
 struct GlobalPipe {
@@ -612,7 +614,7 @@ struct GlobalPipe {
     struct Stage {
         alignas(16) uint32_t hit[kChunk][32 * J];
         uint64_t cl[kChunk];      // cost x L
-        uint64_t w0[32 * J];      // loads at the chunk's start
+        uint64_t w0[kChunk / 32][32 * J];   // loads at the start of each 32 requests
         uint64_t wk[kChunk];      // work that the request adds to the chosen instance
         uint32_t hmax[kChunk];    // 0xFFFFFFFF: no affinity
         uint32_t ch[kChunk];      // list index chosen
@@ -701,51 +703,78 @@ __global__ void __launch_bounds__(GlobalPipe<J>::kThreads, 1) k_choice_all(DevSt
         }
     };
 
-    // one chunk with 31-bit loads and work; w: this lane's loads, moved on
+    // one chunk with loads (as offsets from lo) and work in 31 bits; w: this
+    // lane's loads, moved on.  kPack: they leave room for the list index below
+    // them, so the minimum over the warp is the choice itself; otherwise a vote
+    // finds the lowest lane that holds the minimum.
     constexpr uint32_t kNever = 0x80000000u;
-    auto decide32 = [&](auto kind, Stage &S, uint32_t m, uint32_t (&w)[J]) {
+    constexpr uint32_t kIndexBits = J == 2 ? 6 : J == 4 ? 7 : J == 8 ? 8 : 9;
+    auto decide32 = [&](auto kind, auto pack, Stage &S, uint32_t m, uint32_t (&w)[J], uint64_t lo) {
         constexpr uint32_t kRule = decltype(kind)::value;
+        constexpr bool kPack = decltype(pack)::value;
+        constexpr uint32_t kShift = kPack ? kIndexBits : 0;
         struct alignas(J >= 4 ? 16 : 8) Hits {
             uint32_t v[J];
         };
-        const uint32_t c32 = (uint32_t)cost;
+        const uint32_t c32 = (uint32_t)cost << kShift;
+        if constexpr (kPack) {
+#pragma unroll
+            for (uint32_t j = 0; j < J; ++j)   // past the list: above every key that may win
+                w[j] = w[j] == kNever ? kNever : w[j] << kShift | (lane * J + j);
+        }
         // the next request's staged values, read while this one is decided
         Hits h = *reinterpret_cast<const Hits *>(&S.hit[0][lane * J]);
-        uint32_t cl = (uint32_t)S.cl[0], hm = S.hmax[0];
+        uint32_t cl = (uint32_t)S.cl[0] << kShift, hm = S.hmax[0];
         for (uint32_t rr = 0; rr < m; ++rr) {
-            uint32_t u[J], add[J];   // its work on each instance; what its key adds to the load
-            bool out[J];             // Preble's affinity leaves the instance out
+            if ((rr & 31u) == 0) {
+#pragma unroll
+                for (uint32_t j = 0; j < J; ++j)
+                    if (lane * J + j < nl) S.w0[rr / 32][lane * J + j] = lo + (w[j] >> kShift);
+            }
+            uint32_t u[J], key[J];   // its work on each instance; its keys
 #pragma unroll
             for (uint32_t j = 0; j < J; ++j) {
                 u[j] = cl - c32 * h.v[j];
-                out[j] = kRule == DM_RULE_PREBLE && hm != 0xFFFFFFFFu && h.v[j] != hm;
-                add[j] = kRule == DM_RULE_LEAST_LOADED || (kRule == DM_RULE_PREBLE && hm != 0xFFFFFFFFu) ? 0u : u[j];
+                const bool affine = kRule == DM_RULE_PREBLE && hm != 0xFFFFFFFFu;
+                key[j] = w[j] + (kRule == DM_RULE_LEAST_LOADED || affine ? 0u : u[j]);
+                if (affine && h.v[j] != hm) key[j] = 0xFFFFFFFFu;   // left out
             }
             const uint32_t nx = min(rr + 1, m - 1);
             h = *reinterpret_cast<const Hits *>(&S.hit[nx][lane * J]);
-            cl = (uint32_t)S.cl[nx];
+            cl = (uint32_t)S.cl[nx] << kShift;
             hm = S.hmax[nx];
-            uint32_t bk[J], bj[J];
+            if constexpr (kPack) {
+                uint32_t best = key[0];
 #pragma unroll
-            for (uint32_t j = 0; j < J; ++j) {
-                bk[j] = out[j] ? 0xFFFFFFFFu : w[j] + add[j];
-                bj[j] = j;
+                for (uint32_t j = 1; j < J; ++j) best = min(best, key[j]);
+                best = __reduce_min_sync(0xffffffffu, best);
+#pragma unroll
+                for (uint32_t j = 0; j < J; ++j) w[j] += key[j] == best ? u[j] : 0u;   // keys differ in their index
+                // (least loaded, affinity: the key is the load and its index; else the work lies above the index)
+                if (lane == 0) S.ch[rr] = best & ((1u << kIndexBits) - 1u);
+            } else {
+                uint32_t bj[J];
+#pragma unroll
+                for (uint32_t j = 0; j < J; ++j) bj[j] = j;
+#pragma unroll
+                for (uint32_t s = 1; s < J; s *= 2)   // ties: the lower index
+#pragma unroll
+                    for (uint32_t j = 0; j + s < J; j += 2 * s) {
+                        const bool less = key[j + s] < key[j];
+                        key[j] = less ? key[j + s] : key[j];
+                        bj[j] = less ? bj[j + s] : bj[j];
+                    }
+                const uint32_t kmin = __reduce_min_sync(0xffffffffu, key[0]);
+                const uint32_t eq = __ballot_sync(0xffffffffu, key[0] == kmin);
+                const uint32_t won = eq & (0u - eq) & (1u << lane) ? bj[0] : J;   // the lowest lane's index
+#pragma unroll
+                for (uint32_t j = 0; j < J; ++j) w[j] += won == j ? u[j] : 0u;
+                if (won < J) S.ch[rr] = lane * J + won;
             }
-#pragma unroll
-            for (uint32_t s = 1; s < J; s *= 2)   // ties: the lower index
-#pragma unroll
-                for (uint32_t j = 0; j + s < J; j += 2 * s) {
-                    const bool less = bk[j + s] < bk[j];
-                    bk[j] = less ? bk[j + s] : bk[j];
-                    bj[j] = less ? bj[j + s] : bj[j];
-                }
-            const uint32_t kmin = __reduce_min_sync(0xffffffffu, bk[0]);
-            const uint32_t eq = __ballot_sync(0xffffffffu, bk[0] == kmin);
-            const uint32_t won = eq & (0u - eq) & (1u << lane) ? bj[0] : J;   // the lowest lane's index
-#pragma unroll
-            for (uint32_t j = 0; j < J; ++j) w[j] += won == j ? u[j] : 0u;
-            if (won < J) S.ch[rr] = lane * J + won;
         }
+#pragma unroll
+        for (uint32_t j = 0; j < J; ++j)
+            if (lane * J + j < nl) W[lane * J + j] = lo + (w[j] >> kShift);
     };
 
     auto decide = [&](uint32_t buf, uint32_t m) {
@@ -758,7 +787,6 @@ __global__ void __launch_bounds__(GlobalPipe<J>::kThreads, 1) k_choice_all(DevSt
             const uint32_t x = lane * J + j;
             w64[j] = x < nl ? W[x] : ~0ull;
             if (x < nl) {
-                S.w0[x] = w64[j];
                 lo = min(lo, w64[j]);
                 hi = max(hi, w64[j]);
             }
@@ -778,15 +806,19 @@ __global__ void __launch_bounds__(GlobalPipe<J>::kThreads, 1) k_choice_all(DevSt
             uint32_t w[J];   // past the list: above every key that may win
 #pragma unroll
             for (uint32_t j = 0; j < J; ++j) w[j] = lane * J + j < nl ? (uint32_t)(w64[j] - lo) : kNever;
-            if (rule == DM_RULE_MIN_TTFT) decide32(std::integral_constant<uint32_t, DM_RULE_MIN_TTFT>{}, S, m, w);
-            else if (rule == DM_RULE_LEAST_LOADED)
-                decide32(std::integral_constant<uint32_t, DM_RULE_LEAST_LOADED>{}, S, m, w);
-            else decide32(std::integral_constant<uint32_t, DM_RULE_PREBLE>{}, S, m, w);
-#pragma unroll
-            for (uint32_t j = 0; j < J; ++j)
-                if (lane * J + j < nl) W[lane * J + j] = lo + w[j];
+            auto by_rule = [&](auto pack) {
+                if (rule == DM_RULE_MIN_TTFT)
+                    decide32(std::integral_constant<uint32_t, DM_RULE_MIN_TTFT>{}, pack, S, m, w, lo);
+                else if (rule == DM_RULE_LEAST_LOADED)
+                    decide32(std::integral_constant<uint32_t, DM_RULE_LEAST_LOADED>{}, pack, S, m, w, lo);
+                else decide32(std::integral_constant<uint32_t, DM_RULE_PREBLE>{}, pack, S, m, w, lo);
+            };
+            if (hi - lo + work < (kNever >> kIndexBits)) by_rule(std::true_type{});
+            else by_rule(std::false_type{});
         } else {
             for (uint32_t rr = 0; rr < m; ++rr) {
+                if ((rr & 31u) == 0)
+                    for (uint32_t x = lane; x < nl; x += 32) S.w0[rr / 32][x] = Wv[x];
                 const uint64_t cl = S.cl[rr];
                 const uint32_t hm = S.hmax[rr];
                 // smallest (key, list index): three 32-bit reductions give the exact pair
@@ -826,17 +858,18 @@ __global__ void __launch_bounds__(GlobalPipe<J>::kThreads, 1) k_choice_all(DevSt
         const uint32_t nbr = valid ? d.r_nblk[r] : 0, h = valid ? S.hit[k][x] : 0;
         const uint64_t wk = valid ? S.cl[k] - cost * h : 0;
         if (valid) S.wk[k] = wk;
+        const uint32_t L = valid ? d.r_L[r] : 0, c1 = valid ? d.r_c1[r] : 0, c2 = valid ? d.r_c2[r] : 0;
+        const uint32_t f1 = valid ? d.r_m1[r] : 0, f2 = valid ? d.r_m2[r] : 0;
+        const uint32_t ch = valid ? live[x] : live[0], qh = d.q_head[ch];
         // (its barriers also order the chunk's wk before the sums below)
         const uint64_t pt =
             record_place<kChunk>(PT, x, (uint64_t(nbr) << 32) + 1, valid, k / 32, (m + 31) / 32, lane);
         if (!valid) return;
-        const uint32_t ch = live[x], L = d.r_L[r], c1 = d.r_c1[r], c2 = d.r_c2[r];
-        const uint32_t h1 = hit_tokens(d.r_m1[r], nbr, d.B), h2 = hit_tokens(d.r_m2[r], nbr, d.B);
+        const uint32_t h1 = hit_tokens(f1, nbr, d.B), h2 = hit_tokens(f2, nbr, d.B);
         // the loads as the request found them
-        const uint32_t x1 = inv[c1], x2 = inv[c2];
-        uint64_t wc = S.w0[x], w1 = S.w0[x1], w2 = S.w0[x2];
-        for (uint32_t q = 0; q < (k | 31u); ++q) {
-            if (q >= k) continue;
+        const uint32_t x1 = inv[c1], x2 = inv[c2], q0 = k & ~31u;
+        uint64_t wc = S.w0[q0 / 32][x], w1 = S.w0[q0 / 32][x1], w2 = S.w0[q0 / 32][x2];
+        for (uint32_t q = q0; q < k; ++q) {
             const uint32_t cq = S.ch[q];
             const uint64_t wq = S.wk[q];
             wc += cq == x ? wq : 0;
@@ -855,7 +888,7 @@ __global__ void __launch_bounds__(GlobalPipe<J>::kThreads, 1) k_choice_all(DevSt
         ms.est += wc + wk <= slo;
         if (t1 > slo && t2 > slo) d.info->both_over = 1;
         const uint32_t slot = (uint32_t)pt;
-        if (slot - d.q_head[ch] >= d.Q) {
+        if (slot - qh >= d.Q) {
             set_err(d.err, DM_ERR_CAPACITY);
             return;
         }

@@ -66,3 +66,13 @@ def test_d_choice_ranges(d, cost):
         gpu.commit()
     assert gpu.last_error() == 0 and np.array_equal(gpu.loads(), ora.loads())
     gpu.close()
+
+
+@pytest.mark.parametrize("rule,M", [(6, 64), (7, 64), (8, 64), (7, 128), (8, 250), (7, 400)])
+@pytest.mark.parametrize("cost", [1 << 10, 1 << 14, 1 << 19])
+def test_cluster_choice_ranges(rule, M, cost):
+    # loads and work below 2^31 but no longer beside the list index, then past 2^31
+    tr = _trace(cost, batch=130, n_instances=min(M, 40), vnodes=4)
+    p = Pair(tr.cfg, max_instances=M, max_batch_tokens=1 << 20, max_touch=1 << 13, max_queue=1024, choice_rule=rule)
+    run_trace(p, tr)
+    p.gpu.close()
