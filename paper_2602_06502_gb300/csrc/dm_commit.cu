@@ -84,8 +84,7 @@ __device__ __forceinline__ uint64_t touch_resolve(Slot *t, uint64_t mask, uint64
             return pos_max(&t[i], p1);
         }
         Slot sn[kGroup];
-#pragma unroll
-        for (int j = 0; j < (int)kGroup; ++j) sn[j] = load_slot(t + R + j);
+        load_bucket(t + R, sn);
         uint32_t best = kGroup;
         Slot bs{0, 0};
 #pragma unroll

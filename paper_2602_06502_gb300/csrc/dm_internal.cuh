@@ -419,6 +419,15 @@ __device__ __forceinline__ Slot load_slot(const Slot *p) {
     return s;
 }
 
+// A whole bucket (128-byte aligned), two slots a load.
+__device__ __forceinline__ void load_bucket(const Slot *b, Slot (&s)[kGroup]) {
+#pragma unroll
+    for (int j = 0; j < (int)kGroup; j += 2)
+        asm volatile("ld.global.cg.v4.u64 {%0, %1, %2, %3}, [%4];"
+                     : "=l"(s[j].key), "=l"(s[j].pos1), "=l"(s[j + 1].key), "=l"(s[j + 1].pos1)
+                     : "l"(__cvta_generic_to_global(b + j)));
+}
+
 // Home slot of block b given its group anchor's key.
 __device__ __forceinline__ uint64_t group_home(uint64_t anchor, uint64_t b, uint64_t mask) {
     return (anchor & mask & ~uint64_t(kGroup - 1)) | (b & (kGroup - 1));
@@ -458,8 +467,7 @@ __device__ __forceinline__ uint64_t table_find(const Slot *t, uint64_t mask, uin
     if (loop_limit && loop_limit < walk) walk = loop_limit;
     for (uint64_t nbk = 1; nbk <= walk; ++nbk) {
         Slot sn[kGroup];
-#pragma unroll
-        for (int j = 0; j < (int)kGroup; ++j) sn[j] = load_slot(t + R + j);
+        load_bucket(t + R, sn);
         bool empty = false;
         uint64_t hit = kNoSlot;
         Slot hs{0, 0};
