@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -725,6 +726,29 @@ dm_status dm_route_shard_finish(dm_handle *h, const dm_batch *b, const dm_route_
     return route_finish(h, b, o);
 }
 
+// Whether every output buffer is pinned host memory that the device can write,
+// from its first to its last entry (asked on each call: a buffer may be freed
+// and its address used again); *w: the device addresses.
+static bool host_outputs(const dm_route_out &o, uint32_t n, dm_route_out *w) {
+    *w = o;
+    auto mapped = [n](auto *&p) {
+        using T = std::remove_reference_t<decltype(*p)>;
+        cudaPointerAttributes a{}, z{};
+        unsigned flags = 0;
+        const bool ok = reinterpret_cast<uintptr_t>(p) % sizeof(T) == 0 &&
+                        cudaPointerGetAttributes(&a, p) == cudaSuccess && a.type == cudaMemoryTypeHost &&
+                        cudaPointerGetAttributes(&z, p + n - 1) == cudaSuccess && z.type == cudaMemoryTypeHost &&
+                        a.devicePointer && static_cast<T *>(z.devicePointer) == static_cast<T *>(a.devicePointer) + (n - 1) &&
+                        cudaHostGetFlags(&flags, p) == cudaSuccess &&
+                        !(flags & (cudaHostRegisterReadOnly | cudaHostRegisterIoMemory));
+        if (!ok) cudaGetLastError();
+        else p = static_cast<T *>(a.devicePointer);
+        return ok;
+    };
+    return mapped(w->cand1) && mapped(w->cand2) && mapped(w->hit1) && mapped(w->hit2) && mapped(w->ttft1) &&
+           mapped(w->ttft2) && mapped(w->chosen) && mapped(w->switched);
+}
+
 dm_status dm_route_batch_host_async(dm_handle *h, const dm_batch *b, const dm_route_out *o) {
     dm_status s = check_batch(h, b, o);
     if (s) return s;
@@ -776,12 +800,17 @@ dm_status dm_route_batch_host_async(dm_handle *h, const dm_batch *b, const dm_ro
     if (n) {
         e = cudaEventRecord(x.consumed, h->st);
         x.used = true;
-        struct { void *dst; const void *src; size_t bytes; } cp[] = {
-            {o->cand1, x.out.cand1, n * 4ull}, {o->cand2, x.out.cand2, n * 4ull}, {o->hit1, x.out.hit1, n * 4ull},
-            {o->hit2, x.out.hit2, n * 4ull}, {o->ttft1, x.out.ttft1, n * 8ull}, {o->ttft2, x.out.ttft2, n * 8ull},
-            {o->chosen, x.out.chosen, n * 4ull}, {o->switched, x.out.switched, n * 1ull}};
-        for (auto &c : cp)
-            if (e == cudaSuccess) e = cudaMemcpyAsync(c.dst, c.src, c.bytes, cudaMemcpyDeviceToHost, h->st);
+        dm_route_out w;
+        if (host_outputs(*o, n, &w)) {
+            if (e == cudaSuccess) e = dm::launch_copy_out(x.out, w, n, h->st);
+        } else {
+            struct { void *dst; const void *src; size_t bytes; } cp[] = {
+                {o->cand1, x.out.cand1, n * 4ull}, {o->cand2, x.out.cand2, n * 4ull}, {o->hit1, x.out.hit1, n * 4ull},
+                {o->hit2, x.out.hit2, n * 4ull}, {o->ttft1, x.out.ttft1, n * 8ull}, {o->ttft2, x.out.ttft2, n * 8ull},
+                {o->chosen, x.out.chosen, n * 4ull}, {o->switched, x.out.switched, n * 1ull}};
+            for (auto &c : cp)
+                if (e == cudaSuccess) e = cudaMemcpyAsync(c.dst, c.src, c.bytes, cudaMemcpyDeviceToHost, h->st);
+        }
     }
     return map_cuda(h, e);
 }

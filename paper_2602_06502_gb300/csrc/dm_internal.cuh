@@ -1008,6 +1008,7 @@ cudaError_t launch_adapt_update(const DevState &d, uint64_t *new_set, uint64_t n
 cudaError_t launch_choice(const DevState &d, const dm_route_out &o, uint32_t n, uint64_t seq0,
                           uint64_t t_batch, cudaStream_t st);
 cudaError_t launch_commit(const DevState &d, uint32_t n, cudaStream_t st);
+cudaError_t launch_copy_out(const dm_route_out &o, const dm_route_out &w, uint32_t n, cudaStream_t st);
 cudaError_t launch_rebalance(const DevState &d, uint32_t n, uint64_t seq0, uint32_t call,
                              dm_migration *out, uint32_t cap, uint32_t *n_out, cudaStream_t st);
 cudaError_t launch_hash_keys(const DevState &d, const dm_batch &b, uint64_t *keys, uint64_t *key_off, uint64_t *pos,
