@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(32 + kPotcGen) k_potc(uint32_t n, uint64_t m, 
     const uint32_t pt = tid - 32, j = pt % T, g = pt / T, G = kPotcGen / T;
     auto generate = [&](uint64_t i) {
         if (g >= G || s0 + j >= trials) return;
-        const uint32_t rows = tile * d / 2;
+        const uint32_t rows = ((uint32_t)min((uint64_t)tile, m - i * tile) * d + 1) / 2;   // of its balls
         // state after the increment of choice 0 of row g
         uint64_t z = seed + ((uint64_t(s0 + j) * m + i * tile) * d + 2 * g + 1) * kPhi;
         const uint64_t step = kPhi * (2 * G);
