@@ -26,6 +26,7 @@ namespace dm {
 
 constexpr int kMtThreads = 256;
 constexpr uint32_t kPrepVec = 4;        // requests per thread whose loads the commit prep issues together
+constexpr uint32_t kPrepFan = 512;      // instances up to which its warps keep sums of their own
 constexpr uint32_t kFlagCompact = 1, kFlagRebuild = 2;
 constexpr uint32_t kZeroChunk = 4096;   // slots or flag bytes cleared per chunk
 
@@ -396,8 +397,11 @@ __global__ void __launch_bounds__(kMtThreads) k_maint_a(DevState d) {
 
 __device__ void commit_prep_cta(const DevState &d, uint32_t n, uint64_t *adv);
 
-// n: requests of the batch (for the record layout); dynamic smem: one u64
-// per instance.
+// One u64 per instance, and one per warp and instance where the warps of the
+// commit prep keep sums of their own.
+static size_t prep_smem(uint32_t M) { return sizeof(uint64_t) * M * (M <= kPrepFan ? 1 + kMtThreads / 32 : 1); }
+
+// n: requests of the batch (for the record layout); dynamic smem: prep_smem(M).
 __global__ void __launch_bounds__(kMtThreads) k_maint_c(DevState d, uint32_t n) {
     pdl_enter();
     extern __shared__ __align__(16) unsigned char smem[];
@@ -453,8 +457,10 @@ __global__ void __launch_bounds__(kMtThreads) k_maint_c(DevState d, uint32_t n) 
 // this commit and advance its tail.  The choice kernel already placed every
 // request among its instance's records; only when a rebalance moved a
 // request of this batch are the offsets recomputed (arrival order per final
-// instance), a warp per 32 requests: one thread walking 4,096 requests took
-// 200 us of a rebalanced pass (256 instances, GB300).  One CTA, after every CTA of k_maint_c; adv: one u64 per
+// instance).  4,096 requests on 256 instances, GB300, kernel time: 206 us when
+// one thread walked them, 23 with a warp per 32 requests in turn, 19 with a run
+// of requests and sums of its own per warp (up to kPrepFan instances, whose
+// sums stay below 40 KB).  One CTA, after every CTA of k_maint_c; adv: one u64 per
 // instance in shared memory.
 __device__ void commit_prep_cta(const DevState &d, uint32_t n, uint64_t *adv) {
     for (uint32_t i = threadIdx.x; i < d.M; i += blockDim.x) {
@@ -487,23 +493,71 @@ __device__ void commit_prep_cta(const DevState &d, uint32_t n, uint64_t *adv) {
     if (dirty) {
         __syncthreads();
         for (uint32_t i = threadIdx.x; i < d.M; i += blockDim.x) adv[i] = 0;
-        __syncthreads();
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-        for (uint32_t base = 0; base < n; base += kPrepVec * kMtThreads) {
-            uint32_t f[kPrepVec], nb[kPrepVec];
+        constexpr uint32_t kWarps = kMtThreads / 32;
+        if (d.M <= kPrepFan) {
+            // every warp takes a run of windows, in two passes: its sums per
+            // instance, then, from the sums of the warps before it, the places
+            uint64_t *const mine = adv + uint64_t(wid + 1) * d.M;
+            for (uint32_t i = threadIdx.x; i < kWarps * d.M; i += blockDim.x) adv[d.M + i] = 0;
+            __syncthreads();
+            const uint32_t per = ((n + 31) / 32 + kWarps - 1) / kWarps * 32;   // requests of a warp
+            const uint32_t lo = min(n, wid * per), hi = min(n, lo + per);
+#pragma unroll 1
+            for (int pass = 0; pass < 2; ++pass) {
+                for (uint32_t base = lo; base < hi; base += 32 * kPrepVec) {
+                    uint32_t f[kPrepVec], nb[kPrepVec];
 #pragma unroll
-            for (uint32_t u = 0; u < kPrepVec; ++u) {
-                const uint32_t r = base + u * kMtThreads + threadIdx.x;
-                f[u] = r < n ? d.r_final[r] : 0;
-                nb[u] = r < n ? d.r_nblk[r] : 0;
+                    for (uint32_t u = 0; u < kPrepVec; ++u) {
+                        const uint32_t r = base + 32 * u + lane;
+                        f[u] = r < hi ? d.r_final[r] : 0;
+                        nb[u] = r < hi ? d.r_nblk[r] : 0;
+                    }
+#pragma unroll
+                    for (uint32_t u = 0; u < kPrepVec; ++u) {
+                        const uint32_t r = base + 32 * u + lane;
+                        const bool valid = r < hi;
+                        const uint32_t peers = __match_any_sync(0xffffffffu, valid ? f[u] : 0x80000000u | lane);
+                        const uint64_t sum = peer_sum(peers, nb[u], lane);
+                        const uint64_t p = valid ? mine[f[u]] : 0;
+                        __syncwarp();
+                        if (valid && (peers >> lane) == 1u) mine[f[u]] = p + sum;   // the last of the instance
+                        if (valid && pass) d.r_touchoff[r] = p + sum - nb[u];
+                        __syncwarp();
+                    }
+                }
+                __syncthreads();
+                if (pass == 0) {
+                    for (uint32_t i = threadIdx.x; i < d.M; i += blockDim.x) {
+                        uint64_t run = 0;
+                        for (uint32_t w = 1; w <= kWarps; ++w) {
+                            const uint64_t t = adv[uint64_t(w) * d.M + i];
+                            adv[uint64_t(w) * d.M + i] = run;
+                            run += t;
+                        }
+                        adv[i] = run;
+                    }
+                    __syncthreads();
+                }
             }
+        } else {
+            __syncthreads();
+            for (uint32_t base = 0; base < n; base += kPrepVec * kMtThreads) {
+                uint32_t f[kPrepVec], nb[kPrepVec];
 #pragma unroll
-            for (uint32_t u = 0; u < kPrepVec; ++u) {
-                const uint32_t b0 = base + u * kMtThreads;
-                if (b0 >= n) break;
-                const uint32_t r = b0 + threadIdx.x, m = min(uint32_t(kMtThreads), n - b0);
-                const uint64_t off = record_place<kMtThreads>(adv, f[u], nb[u], r < n, wid, (m + 31) / 32, lane);
-                if (r < n) d.r_touchoff[r] = off;
+                for (uint32_t u = 0; u < kPrepVec; ++u) {
+                    const uint32_t r = base + u * kMtThreads + threadIdx.x;
+                    f[u] = r < n ? d.r_final[r] : 0;
+                    nb[u] = r < n ? d.r_nblk[r] : 0;
+                }
+#pragma unroll
+                for (uint32_t u = 0; u < kPrepVec; ++u) {
+                    const uint32_t b0 = base + u * kMtThreads;
+                    if (b0 >= n) break;
+                    const uint32_t r = b0 + threadIdx.x, m = min(uint32_t(kMtThreads), n - b0);
+                    const uint64_t off = record_place<kMtThreads>(adv, f[u], nb[u], r < n, wid, (m + 31) / 32, lane);
+                    if (r < n) d.r_touchoff[r] = off;
+                }
             }
         }
         __syncthreads();
@@ -938,12 +992,13 @@ static int evict_grid() {
 
 cudaError_t launch_commit(const DevState &d, uint32_t n, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    const size_t smem_a = plan_smem(d.M), smem_c = sizeof(uint64_t) * d.M;
+    const size_t smem_a = plan_smem(d.M), smem_c = prep_smem(d.M);
     static size_t configured = 0;
-    if (smem_a > configured) {   // smem_a > smem_c
+    if (smem_a > configured) {   // (up to kPrepFan instances k_maint_c takes more than for somewhat more of them)
+        const size_t most_c = smem_c > prep_smem(kPrepFan) ? smem_c : prep_smem(kPrepFan);
         cudaError_t e = cudaFuncSetAttribute(k_maint_a, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_a);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_maint_c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_c);
+            e = cudaFuncSetAttribute(k_maint_c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most_c);
         if (e != cudaSuccess) return e;
         configured = smem_a;
     }

@@ -695,18 +695,10 @@ __device__ __forceinline__ void drain_queue(const DevState &d, uint32_t i, uint6
 }
 
 // ---------------------------------------------------------------------------
-// Running sums per instance over a chunk of requests in arrival order: returns
-// PT[ch] as the request finds it and moves it on by `step` (the choice counts
-// records of this batch << 32 | queue tail, so its step is (the request's
-// blocks << 32) + 1).  Called by the kChunk threads of one chunk, a warp per
-// window of 32 requests, in window order over a barrier of their own (valid:
-// the lane has a request; PT in shared memory).
-template <uint32_t kChunk>
-__device__ __forceinline__ uint64_t record_place(uint64_t *PT, uint32_t ch, uint64_t step, bool valid,
-                                                 uint32_t window, uint32_t windows, int lane) {
-    const uint32_t peers = __match_any_sync(0xffffffffu, valid ? ch : 0x80000000u | lane);
+// Inclusive sum of `step` over the lanes of `peers` (which holds this lane) up
+// to this one, by pointer jumping.  Whole warp.
+__device__ __forceinline__ uint64_t peer_sum(uint32_t peers, uint64_t step, int lane) {
     const uint32_t lower = peers & ((1u << lane) - 1u);
-    // inclusive sum over the peers up to this lane, by pointer jumping
     int prev = lower ? 31 - __clz(lower) : -1;
     uint64_t sum = step;
 #pragma unroll
@@ -718,6 +710,20 @@ __device__ __forceinline__ uint64_t record_place(uint64_t *PT, uint32_t ch, uint
             prev = pp;
         }
     }
+    return sum;
+}
+
+// Running sums per instance over a chunk of requests in arrival order: returns
+// PT[ch] as the request finds it and moves it on by `step` (the choice counts
+// records of this batch << 32 | queue tail, so its step is (the request's
+// blocks << 32) + 1).  Called by the kChunk threads of one chunk, a warp per
+// window of 32 requests, in window order over a barrier of their own (valid:
+// the lane has a request; PT in shared memory).
+template <uint32_t kChunk>
+__device__ __forceinline__ uint64_t record_place(uint64_t *PT, uint32_t ch, uint64_t step, bool valid,
+                                                 uint32_t window, uint32_t windows, int lane) {
+    const uint32_t peers = __match_any_sync(0xffffffffu, valid ? ch : 0x80000000u | lane);
+    const uint64_t sum = peer_sum(peers, step, lane);
     const bool last = (peers >> lane) == 1u;
     uint64_t place = 0;
     for (uint32_t w = 0; w < windows; ++w) {

@@ -16,7 +16,7 @@ def _built():
     lib_ready()
 
 
-@pytest.mark.parametrize("live,batch", [(8, 33), (16, 257), (12, 1025), (300, 2100)])
+@pytest.mark.parametrize("live,batch", [(8, 33), (16, 257), (12, 1025), (300, 2100), (511, 1500), (512, 1500)])
 def test_commit_after_moves(live, batch):
     # few virtual nodes: some instances own many prefixes, and a request's other candidate may be far less loaded
     w = workload("tiny", n_instances=live, vnodes=2, slo_us=100_000_000, n_prefix=60, zipf_s=1.2, rho=1.0,
