@@ -460,8 +460,8 @@ __global__ void __launch_bounds__(kMtThreads) k_maint_c(DevState d, uint32_t n) 
 // instance).  4,096 requests on 256 instances, GB300, kernel time: 206 us when
 // one thread walked them, 23 with a warp per 32 requests in turn, 19 with a run
 // of requests and sums of its own per warp (up to kPrepFan instances, whose
-// sums stay below 40 KB).  One CTA, after every CTA of k_maint_c; adv: one u64 per
-// instance in shared memory.
+// sums stay below 40 KB).  One CTA, after every CTA of k_maint_c; adv:
+// prep_smem(M) bytes of shared memory.
 __device__ void commit_prep_cta(const DevState &d, uint32_t n, uint64_t *adv) {
     for (uint32_t i = threadIdx.x; i < d.M; i += blockDim.x) {
         const uint32_t fl = d.mt_flags[i];
