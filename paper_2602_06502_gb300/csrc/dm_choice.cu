@@ -23,6 +23,7 @@
 #include <type_traits>
 
 #include "dm_internal.cuh"
+#include "dm_run_end.h"
 
 namespace dm {
 
@@ -559,28 +560,14 @@ __global__ void __launch_bounds__(kAllBlock, 4) k_probe_all(DevState d, uint32_t
             };
             const uint64_t key0 = cache_key(pl[0] + d.seg_carry[s0], d.Sc), home0 = group_home(key0, 0, mask);
             if (resident_at(t, mask, key0, home0, front, load_slot(t + home0), d.err, d.loop_limit)) {
-                uint32_t lo = 0, hi = nblk;   // block lo is resident; hi is not, or the prompt's end
                 const uint32_t g = max(min(d.r_m1[r], nblk), min(d.r_m2[r], nblk));   // first miss on a candidate
-                uint32_t b[3] = {max(g, 1u) - 1, min(g, nblk - 1), nblk / 2};
-                if (g == 0) b[0] = nblk / 4;
-                if (b[2] < b[0]) b[2] = b[0];
-                while (hi - lo > 1) {
+                RunEnd end(nblk, g);
+                while (end.open()) {
                     bool in[3];
-                    resident(b, in);
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) {   // the resident blocks are a leading run: any order of the three
-                        if (in[q]) lo = max(lo, b[q]);
-                        else hi = min(hi, b[q]);
-                    }
-                    const uint32_t step = (hi - lo) / 4, rest = (hi - lo) & 3u;
-                    b[0] = lo + step + (rest > 2);
-                    b[1] = lo + 2 * step + (rest > 1);
-                    b[2] = min(hi - 1, lo + 3 * step + rest);
-                    b[0] = max(b[0], lo + 1);
-                    b[1] = max(b[1], b[0]);
-                    b[2] = max(b[2], b[1]);
+                    resident(end.b, in);
+                    end.narrow(in);
                 }
-                h = hi;
+                h = end.hi;
             }
         }
         d.h_all[uint64_t(r) * d.M + i] = h * d.B;
