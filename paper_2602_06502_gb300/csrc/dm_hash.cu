@@ -591,6 +591,7 @@ __device__ __noinline__ bool route_task(const DevState &d, const uint32_t *token
             d.r_tcarry[r] = hc;
             tail = tail_done(d, r, nseg, 1);
         }
+        __syncwarp();   // lane 0's values above, before the other lanes read them
         if (__shfl_sync(0xffffffffu, tail, 0)) tail_task(d, r, lane);
     }
     return true;
@@ -968,6 +969,7 @@ __global__ void __launch_bounds__(HP<U>::kThreads, kMinBlocks) k_hash_probe(cons
         constexpr uint32_t kIdleLimit = 1u << 22;
         for (uint32_t idle = 0;;) {
             uint64_t e = lane == 0 ? q_pop(q) : 0;
+            __syncwarp();   // what lane 0 saw when it took the entry (a shuffle orders no memory)
             e = shfl_u64(e, 0);
             if (e == 0) {
                 // done once the hashing warps are done, no warp holds a task

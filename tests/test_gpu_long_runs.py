@@ -55,3 +55,31 @@ def test_run_past_the_head(B, adapt):
     p.check_state(tag="end")
     assert p.hit_tokens > 0
     p.gpu.close()
+
+
+def test_many_runs_past_the_head_at_once():
+    """Runs past the head in every request of a batch, settled by whichever
+    warp completes them: candidates, first misses and carries change with every
+    batch in every place, so a value left from the batch before would show."""
+    B, n, per = 4, 48, 12
+    total = HEAD + 3 * ROUND // 4
+    w = workload("tiny", n_instances=7, block_tokens=B, vnodes=16, capacity=1 << 17, batch=n)
+    p = Pair(w, max_batch_tokens=n * (total + 8) * B, max_touch=n * total, max_queue=4096)
+    for i in range(7):
+        p.add(i)
+    rng = np.random.default_rng(23)
+    docs = [rng.integers(0, 32000, total * B, dtype=np.uint32) for _ in range(per)]
+    for t in range(8):
+        prompts = []
+        for _ in range(n if t else per):
+            k = int(rng.integers(per))
+            cut = int(rng.integers(HEAD - 64, total + 1))
+            own = rng.integers(0, 32000, int(rng.integers(0, 3 * 64)) * B, dtype=np.uint32)
+            prompts.append(np.concatenate([docs[k][:cut * B], own])[:total * B])
+        lens = np.array([len(x) for x in prompts], np.uint32)
+        off = (np.cumsum(lens) - lens).astype(np.uint64)
+        p.route(np.concatenate(prompts), off, lens, 100_000_000 * (t + 1), tag=f"batch {t}")
+        p.commit()
+    p.check_state(tag="end")
+    assert p.hit_tokens > 0
+    p.gpu.close()
