@@ -844,6 +844,8 @@ __device__ __forceinline__ void leading_runs(const int (&st)[F][K], const Slot *
             any |= u[f][q];
         }
     }
+    uint64_t walk = (mask >> 3) + kLinearBuckets + 1;   // buckets of a lookup, as in table_find (at least three)
+    if (loop_limit && loop_limit < walk) walk = loop_limit;
     constexpr uint32_t kPer = F == 2 ? 4 : 8;   // lookups of an instance in a round
     const int g = lane >> 3, gbase = lane & 24;
     while (any) {
@@ -894,22 +896,22 @@ __device__ __forceinline__ void leading_runs(const int (&st)[F][K], const Slot *
         for (int x = 0; x < 2; ++x) {
             const int f = F == 2 ? x : 0;
             const uint64_t fr = front[f];
-            int r = look_bucket(s0[x], k[x], fr, gbase);
+            const int r0 = look_bucket(s0[x], k[x], fr, gbase);
             const int r1 = look_bucket(s1[x], k[x], fr, gbase), r2 = look_bucket(s2[x], k[x], fr, gbase);
-            r = r != kOpen ? r : r1 != kOpen ? r1 : r2;
-            const uint64_t walk = (mask >> 3) + kLinearBuckets + 1;
+            int r = r0 != kOpen || walk < 2 ? r0 : r1 != kOpen || walk < 3 ? r1 : r2;
             for (uint64_t j = 3; __any_sync(0xffffffffu, r == kOpen); ++j) {   // (no lookup: found room)
                 const bool open = r == kOpen;
+                if (j >= walk) {
+                    if (open) {
+                        set_err(err, DM_ERR_TIMEOUT);
+                        r = kOut;
+                    }
+                    break;
+                }
                 Slot sj{0, 0};
                 if (open) sj = load_slot(t[f] + probe_bucket(j, R0[x], k[x], mask) + (lane & 7));
                 const int rj = look_bucket(sj, k[x], fr, gbase);
                 if (open) r = rj;
-                if (j > walk || (loop_limit && j > loop_limit)) {
-                    if (r == kOpen) {
-                        set_err(err, DM_ERR_TIMEOUT);
-                        r = kOut;
-                    }
-                }
             }
             outs[x] = __ballot_sync(0xffffffffu, has[x] && r == kOut);
         }

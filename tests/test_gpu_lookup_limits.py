@@ -1,7 +1,10 @@
 """Index lookups that reach the limit of their bucket walk
-(`test_loop_limit`) and end the call in a sticky DM_ERR_TIMEOUT.  A group of 8
-blocks committed after another one with the same home bucket lies in the second
-bucket of its probe order."""
+(`test_loop_limit`): a lookup looks into that many buckets of its key's probe
+order and no more, and one still open then ends the call in a sticky
+DM_ERR_TIMEOUT.  Prompts of whole bucket groups (8 blocks) with the same home
+bucket are routed and committed one after the other, so that the second group
+lies in the second bucket of its order and each key of the third one in its
+third."""
 
 import numpy as np
 import pytest
@@ -79,6 +82,33 @@ def _search(rng, blocks, s, ok):
         if ok(*i):
             return p, i
     raise AssertionError("no such prompt")
+
+
+@pytest.mark.parametrize("limit", [0, 1, 2, 3])
+def test_routing_lookup_limit(limit):
+    from paper_2602_06502_gb300 import dualmap as D
+    s = Sides(limit, 5, 4)   # rule 5: always the first candidate
+    rng = np.random.default_rng(3)
+    first, (h, _, _, c1) = _search(rng, 8, s, lambda *a: True)
+    home, prompts = h[0], [first]
+    taken = {bucket(0, home, 0), bucket(1, home, 0)}
+    while len(prompts) < 3:
+        prompts.append(_search(rng, 8, s, lambda g, keys, _, c: g[0] == home and c == c1 and
+                               not taken & {bucket(2, home, k) for k in keys})[0])
+    # prompt k is new and finds the first k buckets of its order full; then it is in bucket k
+    for k, p in enumerate(prompts + prompts):
+        want, got = s.route([p])
+        if limit and k % 3 >= limit:
+            assert s.gpu.last_error() == D.DM_ERR_TIMEOUT
+            assert D.dm_commit_cache(s.gpu.h) == D.DM_ERR_TIMEOUT
+            break
+        assert s.gpu.last_error() == 0
+        assert want["hit1"][0] == (8 * B if k >= 3 else 0)
+        for f in OUT_KEYS:
+            assert np.array_equal(got[f].astype(want[f].dtype), want[f]), (k, f)
+        s.commit()
+    assert k == (limit if limit in (1, 2) else 5)
+    s.gpu.close()
 
 
 @pytest.mark.parametrize("limit", [0, 1])
