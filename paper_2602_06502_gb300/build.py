@@ -44,7 +44,7 @@ def build(force=False, verbose=False, extra=(), debug=False):
     if debug:
         extra = ("-DDM_DEBUG",) + tuple(extra)
     os.makedirs(bdir, exist_ok=True)
-    headers = [os.path.join(CSRC, h) for h in ("dm_internal.cuh", "dm_run_end.h")]
+    headers = [os.path.join(CSRC, h) for h in ("dm_internal.cuh", "dm_launch.h", "dm_run_end.h")]
     headers.append(os.path.join(ROOT, "include", "dualmap.h"))
     objs, jobs = [], []
     for s in SOURCES:

@@ -20,6 +20,7 @@
 //
 // At the end of the file: routing with d candidates (App. A.8).
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "dm_internal.cuh"
@@ -974,11 +975,8 @@ template <uint32_t J>
 static cudaError_t launch_choice_all(const DevState &d, const dm_route_out &o, uint32_t n, uint64_t seq0,
                                      uint64_t t_batch, cudaStream_t st) {
     const size_t smem = GlobalPipe<J>::smem(d.M);
-    static size_t configured = 0;
-    if (smem > configured) {
-        DM_TRY(cudaFuncSetAttribute(k_choice_all<J>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        configured = smem;
-    }
+    static SmemOptIn opt;
+    DM_TRY(opt_in_smem(opt, smem, k_choice_all<J>));
     return launch_pdl(k_choice_all<J>, 1, GlobalPipe<J>::kThreads, smem, st, d, o, n, seq0, t_batch);
 }
 
@@ -1170,33 +1168,30 @@ cudaError_t launch_choice(const DevState &d, const dm_route_out &o, uint32_t n, 
         else if (d.M <= 512) DM_TRY(launch_choice_all<16>(d, o, n, seq0, t_batch, st));
         else {
             // as much shared memory as the device allows, up to what 1024 requests need
-            static uint32_t smem_g = 0, smem_M = 0;
-            if (smem_M != d.M) {
-                int dev = 0, optin = 0;
+            static SmemOptIn opt;
+            static std::atomic<uint32_t> rooms[kDevices];
+            int dev = 0;
+            DM_TRY(cudaGetDevice(&dev));
+            if (dev < 0 || dev >= kDevices) return cudaErrorInvalidDevice;
+            uint32_t room = rooms[dev].load(std::memory_order_relaxed);
+            if (!room) {
+                int optin = 0;
                 cudaFuncAttributes fa{};
-                DM_TRY(cudaGetDevice(&dev));
                 DM_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
                 DM_TRY(cudaFuncGetAttributes(&fa, k_choice_global));
-                const size_t want = global_stage_off(d.M) + size_t(kGlobalReqMax) * (kGlobalReqBytes + 4ull * d.M);
-                const size_t room = size_t(optin) - fa.sharedSizeBytes;
-                smem_g = (uint32_t)(want < room ? want : room);
-                DM_TRY(cudaFuncSetAttribute(k_choice_global, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)smem_g));
-                smem_M = d.M;
+                room = (uint32_t)(size_t(optin) - fa.sharedSizeBytes);
+                rooms[dev].store(room, std::memory_order_relaxed);
             }
+            const size_t want = global_stage_off(d.M) + size_t(kGlobalReqMax) * (kGlobalReqBytes + 4ull * d.M);
+            const uint32_t smem_g = (uint32_t)std::min<size_t>(want, room);
+            DM_TRY(opt_in_smem(opt, smem_g, k_choice_global));
             DM_TRY(launch_pdl(k_choice_global, 1, 1024, smem_g, st, d, o, n, seq0, t_batch, smem_g));
         }
         return cudaGetLastError();
     }
     const size_t smem = choice_smem(d.M);
-    static size_t configured = 0;
-    if (smem > configured) {
-        for (auto k : {k_choice<false>, k_choice<true>}) {
-            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-        configured = smem;
-    }
+    static SmemOptIn opt;
+    DM_TRY(opt_in_smem(opt, smem, k_choice<false>, k_choice<true>));
     // CTA 0 decides; CTAs 1.. sum the batch's segment carries meanwhile (a warp per request)
     constexpr unsigned threads = Pipe<kChoiceChunk>::kThreads, per = threads / 32;
     const unsigned grid = 1 + std::min((n + per - 1) / per, 2u * 152u);
@@ -1704,11 +1699,8 @@ static cudaError_t launch_choice_d(const DevState &d, const dm_route_out_d &o, u
                                    uint64_t t_batch, cudaStream_t st) {
     constexpr uint32_t kChunk = choice_d_chunk(ND);
     const size_t smem = size_t(d.M) * 16 + 3 * sizeof(ChoiceStageD<ND, kChunk>);
-    static size_t configured = 0;
-    if (smem > configured) {
-        DM_TRY(cudaFuncSetAttribute(k_choice_d<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        configured = smem;
-    }
+    static SmemOptIn opt;
+    DM_TRY(opt_in_smem(opt, smem, k_choice_d<ND>));
     return launch_pdl(k_choice_d<ND>, 1, Pipe<kChunk>::kThreads, smem, st, d, o, n, seq0, t_batch);
 }
 

@@ -993,15 +993,9 @@ static int evict_grid() {
 cudaError_t launch_commit(const DevState &d, uint32_t n, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     const size_t smem_a = plan_smem(d.M), smem_c = prep_smem(d.M);
-    static size_t configured = 0;
-    if (smem_a > configured) {   // (up to kPrepFan instances k_maint_c takes more than for somewhat more of them)
-        const size_t most_c = smem_c > prep_smem(kPrepFan) ? smem_c : prep_smem(kPrepFan);
-        cudaError_t e = cudaFuncSetAttribute(k_maint_a, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_a);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_maint_c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most_c);
-        if (e != cudaSuccess) return e;
-        configured = smem_a;
-    }
+    static SmemOptIn opt_a, opt_c;
+    DM_TRY(opt_in_smem(opt_a, smem_a, k_maint_a));
+    DM_TRY(opt_in_smem(opt_c, smem_c, k_maint_c));
     // every CTA of k_maint_a computes the plan over all instances: two per SM
     static const int g_a = full_grid(k_maint_a, kMtThreads) < 2 * sm_count() ? full_grid(k_maint_a, kMtThreads)
                                                                                 : 2 * sm_count(),

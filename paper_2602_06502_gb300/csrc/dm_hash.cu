@@ -224,13 +224,12 @@ __global__ void __launch_bounds__(256, 4) k_hash(DevState d, const uint32_t *__r
 
 // Grids of the hashing kernels, per device (SM counts may differ).
 namespace {
-constexpr int kGridDevices = 64;
-std::atomic<int> g_grid[kGridDevices][2];
+std::atomic<int> g_grid[kDevices][2];
 
 template <typename K>
 int grid_for_device(int which, K kernel) {
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kGridDevices) return full_grid(kernel, 256);
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return full_grid(kernel, 256);
     int g = g_grid[dev][which].load(std::memory_order_relaxed);
     if (!g) {
         g = full_grid(kernel, 256);
@@ -1027,10 +1026,10 @@ __global__ void __launch_bounds__(HP<U>::kThreads, kMinBlocks) k_hash_probe(cons
 template <int U, bool kAdapt>
 static cudaError_t launch_hash_probe_u(const DevState &d, const dm_batch &b, uint64_t E, uint32_t r0, uint32_t r1,
                                        cudaStream_t st) {
-    static std::atomic<int> grids[kGridDevices];
+    static std::atomic<int> grids[kDevices];
     int dev = 0;
     DM_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= kGridDevices) return cudaErrorInvalidDevice;
+    if (dev < 0 || dev >= kDevices) return cudaErrorInvalidDevice;
     int grid = grids[dev].load(std::memory_order_relaxed);
     if (!grid) {
         DM_TRY(cudaFuncSetAttribute(k_hash_probe<U, kAdapt>, cudaFuncAttributeMaxDynamicSharedMemorySize,

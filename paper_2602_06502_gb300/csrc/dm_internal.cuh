@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/dualmap.h"
+#include "dm_launch.h"
 
 namespace dm {
 
@@ -324,6 +325,22 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, unsigned bloc
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// Allow kernels that are launched with up to `bytes` of dynamic shared memory
+// that much on the current device.
+template <typename... K>
+inline cudaError_t opt_in_smem(SmemOptIn &opt, size_t bytes, K... kernels) {
+    int dev = 0;
+    DM_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= kDevices) return cudaErrorInvalidDevice;
+    return static_cast<cudaError_t>(opt.raise(dev, bytes, [&] {
+        cudaError_t e = cudaSuccess;
+        ((e = e == cudaSuccess ? cudaFuncSetAttribute(kernels, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)
+                               : e),
+         ...);
+        return static_cast<int>(e);
+    }));
 }
 
 // ---------------------------------------------------------------------------

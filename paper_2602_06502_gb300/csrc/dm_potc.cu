@@ -153,9 +153,8 @@ extern "C" dm_status dm_potc_max_loads(uint32_t n_bins, uint64_t m_balls, uint32
     const auto st = static_cast<cudaStream_t>(stream);
     const auto k = d == 1 ? dm::k_potc<1> : d == 2 ? dm::k_potc<2> : d == 3 ? dm::k_potc<3> : d == 4 ? dm::k_potc<4>
                                                                                                      : dm::k_potc<0>;
-    cudaError_t e = cudaSuccess;
-    if (smem > 16 * 1024)   // past 48 KB with the tiles
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 32 * 1024);
+    static dm::SmemOptIn opt[5];   // past 48 KB with the tiles
+    cudaError_t e = dm::opt_in_smem(opt[d <= 4 ? d : 0], smem, k);
     if (e == cudaSuccess) {
         k<<<grid, 32 + dm::kPotcGen, smem, st>>>(n_bins, m_balls, d, trials, seed, max_load_dev, T, tile);
         e = cudaGetLastError();

@@ -524,13 +524,8 @@ cudaError_t launch_rebalance(const DevState &d, uint32_t n, uint64_t seq0, uint3
         while (sort_cap < 8192 && fixed + rb_sort_bytes(sort_cap * 2) <= budget) sort_cap *= 2;
     }
     const size_t smem = fixed + rb_sort_bytes(sort_cap);
-    static size_t configured = 0;
-    if (smem > configured) {
-        cudaError_t e = cudaFuncSetAttribute(k_rebalance, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-        configured = smem;
-    }
+    static SmemOptIn opt;
+    DM_TRY(opt_in_smem(opt, smem, k_rebalance));
     DM_TRY(launch_pdl(k_rebalance, 1, 1024, smem, st, d, n, seq0, call, out, cap, n_out, sort_cap));
     return cudaGetLastError();
 }

@@ -200,9 +200,8 @@ cudaError_t launch_ring_update(DevState &d, const DevState &next, uint32_t id, b
     uint32_t P = 1;
     while (P < d.V) P <<= 1;
     const size_t smem = P <= kSortSmem ? size_t(P) * 12 : 0;
-    constexpr size_t kState = sizeof(uint32_t) * (kMaxInstances / 32);   // state_role's words count too
-    if (smem + kState > 48 * 1024)
-        DM_TRY(cudaFuncSetAttribute(k_gen_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    static SmemOptIn opt;
+    DM_TRY(opt_in_smem(opt, smem, k_gen_sort));   // (state_role's words come on top: past 48 KB from 4,096 entries on)
     DM_TRY(launch_pdl(k_gen_sort, d.nrings + 1, 1024, smem, st, d, id, scratch_pos, scratch_vidx, P,
                       uint8_t(add ? 1 : 2)));
     RingSet rs{};
