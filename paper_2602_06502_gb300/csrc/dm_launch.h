@@ -35,4 +35,16 @@ class SmemOptIn {
     std::atomic<size_t> have_[kDevices] = {};
 };
 
+// Trials per CTA (at most a warp's lanes) of the d-choices sweep, and its CTAs,
+// such that every SM gets the same number of them: 10,000 trials on 152 SMs run
+// as 3 x 152 CTAs of 22.
+struct PotcShape {
+    uint32_t per_cta, grid;
+};
+inline PotcShape potc_shape(uint64_t trials, uint64_t sms) {   // trials >= 1
+    const uint64_t per_sm = (trials + sms * 32 - 1) / (sms * 32);
+    const uint64_t T = (trials + sms * per_sm - 1) / (sms * per_sm);
+    return {(uint32_t)T, (uint32_t)((trials + T - 1) / T)};
+}
+
 }  // namespace dm

@@ -48,14 +48,14 @@ __global__ void __launch_bounds__(32 + kPotcGen) k_potc(uint32_t n, uint64_t m, 
                                                         uint32_t tile) {
     extern __shared__ uint32_t s_load[];   // n x 32 loads
     __shared__ uint32_t s_off[2][kPotcRows][32];
-    const uint32_t tid = threadIdx.x, s0 = blockIdx.x * T;
+    const uint32_t tid = threadIdx.x, s0 = blockIdx.x * T, here = min(T, trials - s0);   // trials of this CTA
     for (uint32_t i = tid; i < n * 32; i += blockDim.x) s_load[i] = 0;
     const uint64_t tiles = (m + tile - 1) / tile;
     constexpr uint64_t kPhi = 0x9E3779B97F4A7C15ull;
     // generating thread: trial j of the CTA, rows g, g + G, ...
     const uint32_t pt = tid - 32, j = pt % T, g = pt / T, G = kPotcGen / T;
     auto generate = [&](uint64_t i) {
-        if (g >= G || s0 + j >= trials) return;
+        if (g >= G || j >= here) return;
         const uint32_t rows = ((uint32_t)min((uint64_t)tile, m - i * tile) * d + 1) / 2;   // of its balls
         // state after the increment of choice 0 of row g
         uint64_t z = seed + ((uint64_t(s0 + j) * m + i * tile) * d + 2 * g + 1) * kPhi;
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(32 + kPotcGen) k_potc(uint32_t n, uint64_t m, 
         return *reinterpret_cast<volatile uint32_t *>(reinterpret_cast<unsigned char *>(s_load) + off);
     };
     auto place = [&](uint64_t i) {   // the CTA's first warp
-        if (tid >= T || s0 + tid >= trials) return;
+        if (tid >= here) return;
         const uint32_t balls = (uint32_t)min((uint64_t)tile, m - i * tile);
         const uint32_t(*const in)[32] = s_off[i & 1];
         uint32_t t = 0;
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(32 + kPotcGen) k_potc(uint32_t n, uint64_t m, 
         else if (i + 1 < tiles) generate(i + 1);
         __syncthreads();
     }
-    if (tid < T && s0 + tid < trials) {
+    if (tid < here) {
         uint32_t mx = 0;
         for (uint32_t b = 0; b < n; ++b) mx = max(mx, s_load[b * 32 + tid]);
         max_load[s0 + tid] = mx;
@@ -142,12 +142,7 @@ extern "C" dm_status dm_potc_max_loads(uint32_t n_bins, uint64_t m_balls, uint32
     if (n_bins < 1 || n_bins > 256 || d < 1 || d > 64 || m_balls > 0xFFFFFFFFull || !max_load_dev)
         return DM_ERR_INVALID_ARG;
     if (trials == 0) return DM_OK;
-    // trials per CTA (at most a warp's lanes) such that every SM gets the
-    // same number of CTAs: 10,000 trials on 152 SMs run as 3 x 152 CTAs of 22
-    const uint32_t sms = (uint32_t)dm::sm_count();
-    const uint32_t per_sm = (trials + sms * 32 - 1) / (sms * 32);
-    const uint32_t T = (trials + sms * per_sm - 1) / (sms * per_sm);
-    const unsigned grid = (trials + T - 1) / T;
+    const dm::PotcShape shape = dm::potc_shape(trials, (uint64_t)dm::sm_count());
     const uint32_t tile = 2 * dm::kPotcRows / d & ~3u;   // d <= 64: at least 4 balls
     const size_t smem = size_t(n_bins) * 32 * 4;         // at most 32 KB
     const auto st = static_cast<cudaStream_t>(stream);
@@ -156,7 +151,8 @@ extern "C" dm_status dm_potc_max_loads(uint32_t n_bins, uint64_t m_balls, uint32
     static dm::SmemOptIn opt[5];   // past 48 KB with the tiles
     cudaError_t e = dm::opt_in_smem(opt[d <= 4 ? d : 0], smem, k);
     if (e == cudaSuccess) {
-        k<<<grid, 32 + dm::kPotcGen, smem, st>>>(n_bins, m_balls, d, trials, seed, max_load_dev, T, tile);
+        k<<<shape.grid, 32 + dm::kPotcGen, smem, st>>>(n_bins, m_balls, d, trials, seed, max_load_dev, shape.per_cta,
+                                                       tile);
         e = cudaGetLastError();
     }
     return e == cudaSuccess ? DM_OK : DM_ERR_CUDA;

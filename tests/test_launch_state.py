@@ -64,6 +64,12 @@ extern "C" int failure_is_not_kept() {
     if (opt.raise(3, 60000, [] { return 700; }) != 700) return 1;
     return opt.raise(3, 60000, [] { return set_to(3, 60000); }) || allowed[3] != 60000 ? 2 : 0;
 }
+
+extern "C" void potc_shape(uint32_t trials, uint32_t sms, uint32_t *per_cta, uint32_t *grid) {
+    const dm::PotcShape s = dm::potc_shape(trials, sms);
+    *per_cta = s.per_cta;
+    *grid = s.grid;
+}
 """
 
 
@@ -79,3 +85,13 @@ def lib(tmp_path_factory):
 @pytest.mark.parametrize("check", ["two_devices", "racing_sizes", "failure_is_not_kept"])
 def test_shared_memory_opt_in(lib, check):
     assert getattr(lib, check)() == 0
+
+
+@pytest.mark.parametrize("trials", [1, 31, 32, 33, 152, 4864, 4865, 10_000, 1 << 31, (1 << 32) - 4864,
+                                    (1 << 32) - 4863, (1 << 32) - 1])
+@pytest.mark.parametrize("sms", [1, 148, 152])
+def test_sweep_shape_covers_every_trial(lib, trials, sms):
+    T, grid = C.c_uint32(), C.c_uint32()
+    lib.potc_shape(trials, sms, C.byref(T), C.byref(grid))
+    assert 1 <= T.value <= 32 and (grid.value - 1) * T.value < trials <= grid.value * T.value
+    assert grid.value < 1 << 31 or sms == 1
