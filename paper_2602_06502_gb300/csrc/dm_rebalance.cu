@@ -212,7 +212,7 @@ __device__ bool scan_hotspot(const DevState &d, uint32_t i, uint32_t tail, uint3
         if (valid && e.moved != kTomb && e.moved != call && e.remaining == e.work) {
             const uint64_t ttft_i = ahead + inc;
             const uint32_t j = e.c1 == i ? e.c2 : e.c1;
-            const uint64_t own = d.cost * (e.L - (j == e.c1 ? e.h1 : e.h2));
+            const uint64_t own = uint64_t(d.cost) * (e.L - (j == e.c1 ? e.h1 : e.h2));
             const uint64_t ttft_j = W[j] + own;
             if ((int64_t)(ttft_i - ttft_j) > 0 && ttft_j < d.slo) now = true;
             const bool earlier = (st[j] & kStHot) && (W[j] > W[i] || (W[j] == W[i] && j < i));
