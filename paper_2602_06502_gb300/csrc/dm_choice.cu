@@ -1194,7 +1194,8 @@ cudaError_t launch_choice(const DevState &d, const dm_route_out &o, uint32_t n, 
     DM_TRY(opt_in_smem(opt, smem, k_choice<false>, k_choice<true>));
     // CTA 0 decides; CTAs 1.. sum the batch's segment carries meanwhile (a warp per request)
     constexpr unsigned threads = Pipe<kChoiceChunk>::kThreads, per = threads / 32;
-    const unsigned grid = 1 + std::min((n + per - 1) / per, 2u * 152u);
+    static const unsigned most = 2 * (unsigned)sm_count();
+    const unsigned grid = 1 + std::min((n + per - 1) / per, most);
     if (d.rule == DM_RULE_DUALMAP)
         DM_TRY(launch_pdl(k_choice<false>, grid, threads, smem, st, d, o, n, seq0, t_batch));
     else
