@@ -731,18 +731,21 @@ dm_status dm_route_shard_finish(dm_handle *h, const dm_batch *b, const dm_route_
 // and its address used again); *w: the device addresses.
 static bool host_outputs(const dm_route_out &o, uint32_t n, dm_route_out *w) {
     *w = o;
-    auto mapped = [n](auto *&p) {
+    auto ask = [](cudaError_t e) {
+        if (e != cudaSuccess) cudaGetLastError();   // an error of the query itself, answered here
+        return e == cudaSuccess;
+    };
+    auto mapped = [n, ask](auto *&p) {
         using T = std::remove_reference_t<decltype(*p)>;
         cudaPointerAttributes a{}, z{};
         unsigned flags = 0;
         const bool ok = reinterpret_cast<uintptr_t>(p) % sizeof(T) == 0 &&
-                        cudaPointerGetAttributes(&a, p) == cudaSuccess && a.type == cudaMemoryTypeHost &&
-                        cudaPointerGetAttributes(&z, p + n - 1) == cudaSuccess && z.type == cudaMemoryTypeHost &&
+                        ask(cudaPointerGetAttributes(&a, p)) && a.type == cudaMemoryTypeHost &&
+                        ask(cudaPointerGetAttributes(&z, p + n - 1)) && z.type == cudaMemoryTypeHost &&
                         a.devicePointer && static_cast<T *>(z.devicePointer) == static_cast<T *>(a.devicePointer) + (n - 1) &&
-                        cudaHostGetFlags(&flags, p) == cudaSuccess &&
+                        ask(cudaHostGetFlags(&flags, p)) &&
                         !(flags & (cudaHostRegisterReadOnly | cudaHostRegisterIoMemory));
-        if (!ok) cudaGetLastError();
-        else p = static_cast<T *>(a.devicePointer);
+        if (ok) p = static_cast<T *>(a.devicePointer);
         return ok;
     };
     return mapped(w->cand1) && mapped(w->cand2) && mapped(w->hit1) && mapped(w->hit2) && mapped(w->ttft1) &&
