@@ -117,9 +117,8 @@ __device__ void finish_metrics(const DevState &d, uint32_t n, MetricSums ms, uns
 // Chunk t is staged while chunk t - 1 is decided and chunk t - 2 emitted,
 // over three staging buffers.  Measured (GB300, kernel time for 4,096 agent
 // prompts, two and four candidates): 191 and 5,200 us with rounds found by
-// votes and with one thread; 123 and 404 us when the deciding warp read and
-// wrote 64-bit loads in shared memory at every level (136 and 400 cycles a
-// level, 780 a window); 88 and 175 us so (84 cycles a level, 470 a window).
+// votes and with one thread, 82 and 164 us so (84 and 200 cycles a level, 470
+// a window).
 constexpr uint8_t kNoLevel = 255;
 
 // The deciding warp has its SM sub-partition to itself (warps are dealt to the
@@ -516,8 +515,7 @@ __global__ void __launch_bounds__(Pipe<kChoiceChunk>::kThreads, 1) k_choice(DevS
 // same block), then by three probes a round, each round leaving a quarter of
 // the range; lanes that probe the same block read the same prefix value.
 // Bound by dependent 16-byte index reads.  4,096 agent prompts x 64
-// instances, GB300: 822 us with a warp per pair testing 32, then 128 blocks a
-// round; 220 us by bisection (ten rounds of one probe); 90 us so.
+// instances, GB300: 822 us with a warp per pair that walked the run, 90 us so.
 constexpr int kAllBlock = 256;
 
 // resident_at past the home slot (not inlined: three of these in a round).
@@ -646,10 +644,7 @@ __global__ void __launch_bounds__(kAllBlock) k_probe_pairs(DevState d, uint32_t 
 // warps add up.
 // 4,096 agent prompts on 64 instances, min TTFT, GB300: 1,678 us with 64-bit
 // keys and loads in shared memory, three reductions a request, and staging
-// and emission between the chunks; 922 us when the deciding warp also read
-// and wrote the loads in shared memory for every request; 302 us with a vote
-// for the winning lane and sums over whole chunks in the emitting warps; 205 us
-// so.
+// and emission between the chunks, 204 us so (100 cycles a request).
 constexpr uint32_t kGlobalStageThreads = 256;
 template <uint32_t J>
 struct GlobalPipe {

@@ -457,11 +457,12 @@ __global__ void __launch_bounds__(kMtThreads) k_maint_c(DevState d, uint32_t n) 
 // this commit and advance its tail.  The choice kernel already placed every
 // request among its instance's records; only when a rebalance moved a
 // request of this batch are the offsets recomputed (arrival order per final
-// instance).  4,096 requests on 256 instances, GB300, kernel time: 206 us when
-// one thread walked them, 23 with a warp per 32 requests in turn, 19 with a run
-// of requests and sums of its own per warp (up to kPrepFan instances, whose
-// sums stay below 40 KB).  One CTA, after every CTA of k_maint_c; adv:
-// prep_smem(M) bytes of shared memory.
+// instance): by a run of requests and sums of its own per warp up to kPrepFan
+// instances (whose sums stay below 40 KB), by a warp per 32 requests in turn
+// above.  4,096 requests on 256 instances, GB300, kernel time: 206 us when one
+// thread walked them, 23 with the warps in turn, 19 with runs (a rebalanced
+// pass 234.0 and 231.4 us, each side's repeats within 0.1 %).  One CTA, after
+// every CTA of k_maint_c; adv: prep_smem(M) bytes of shared memory.
 __device__ void commit_prep_cta(const DevState &d, uint32_t n, uint64_t *adv) {
     for (uint32_t i = threadIdx.x; i < d.M; i += blockDim.x) {
         const uint32_t fl = d.mt_flags[i];
