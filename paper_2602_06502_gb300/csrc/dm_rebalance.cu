@@ -17,7 +17,11 @@
 // Most hotspots have no request that could move (256 instances, 4,096 prompts
 // a batch: 31-38 hotspots, 1-9 moves).  So a warp per hotspot first looks for
 // one under the loads at the call's start, all hotspots at once, and only the
-// hotspots that might move one are visited (scan_hotspot).
+// hotspots that might move one are visited (scan_hotspot).  A warp takes 11 us
+// for 1,024 entries and the whole CTA of a visit 4 for as many or fewer, so a
+// hotspot with more than kScanPer entries for each of the hotspots is visited
+// without a scan (one hotspot of 32,768 entries that cannot move: 351 us when it
+// was scanned too, 122 without).
 #include "dm_internal.cuh"
 
 namespace dm {
@@ -179,11 +183,12 @@ __device__ void bitonic_sort(uint64_t *key, uint64_t *seq, uint64_t *tt, uint32_
 // targets: work moved to a target makes a move to it less likely, so a hotspot
 // without a candidate now has none at its turn unless an earlier hotspot that
 // it would move to has given work away.  Returns whether a request passes the
-// move test now; *later: bit (id & 63) of each earlier hotspot to which a
-// request would move if nothing were queued there.  Whole warp; the next 32
+// move test now; if none does, *later: bit (id & 63) of each earlier hotspot to
+// which a request would move if nothing were queued there.  Whole warp; the next 32
 // entries are loaded while these are tested.
 // Per-instance byte: the instance's state and two flags of this call.
-constexpr uint8_t kStMask = 0x3F, kStHot = 0x80, kStIdle = 0x40;   // hotspot; hotspot with nothing to move now
+constexpr uint8_t kStLive = 1, kStHot = 0x80, kStIdle = 0x40;   // (of the states 0-2 only 1 is odd); hotspot; hotspot with nothing to move now
+constexpr uint32_t kScanPer = 256;
 constexpr uint32_t kLater = 128;   // hotspots (by rank) whose `later` is kept; those after it: any
 struct ScanEntry {
     uint64_t work, remaining;
@@ -219,11 +224,12 @@ __device__ bool scan_hotspot(const DevState &d, uint32_t i, uint32_t tail, uint3
             if (earlier && (int64_t)(ttft_i - own) > 0 && own < d.slo) lt |= 1ull << (j & 63);
         }
         ahead += shfl_u64(inc, 31);
+        if (__any_sync(0xffffffffu, now)) return true;   // visited whatever `later` is
     }
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) lt |= shfl_xor_u64(lt, o);
     *later = lt;
-    return __any_sync(0xffffffffu, now);
+    return false;
 }
 
 // Single CTA of 1024 threads.
@@ -290,7 +296,8 @@ __global__ void __launch_bounds__(1024) k_rebalance(DevState d, uint32_t n, uint
     const uint64_t cost = d.cost;
     for (uint32_t hi = threadIdx.x >> 5; hi < nhot && !fresh; hi += blockDim.x >> 5) {   // fresh hits are probed at the visit
         const uint32_t i = hotl[hi];
-        uint64_t later;
+        if (tails[i] - d.q_head[i] > uint64_t(kScanPer) * nhot) continue;   // visited
+        uint64_t later = 0;
         const bool now = scan_hotspot(d, i, tails[i], call, W, st, threadIdx.x & 31, &later);
         if ((threadIdx.x & 31) == 0) {
             if (!now) st[i] |= kStIdle;
@@ -323,7 +330,7 @@ __global__ void __launch_bounds__(1024) k_rebalance(DevState d, uint32_t n, uint
                 // probe the other candidate's index now, a warp per entry in
                 // turn; the pending batch's own entries keep their stored
                 // hit (no commit since their routing: the same probe)
-                const bool need = elig && (st[jj] & kStMask) == 1 && !(e.seq >= seq0 && e.seq < seq0 + n);
+                const bool need = elig && (st[jj] & kStLive) && !(e.seq >= seq0 && e.seq < seq0 + n);
                 const int lane = threadIdx.x & 31;
                 for (uint32_t m = __ballot_sync(0xffffffffu, need); m; m &= m - 1) {
                     const int src = __ffs(m) - 1;
@@ -429,7 +436,7 @@ __global__ void __launch_bounds__(1024) k_rebalance(DevState d, uint32_t n, uint
                         break;
                     }
                     const uint32_t j = Ch.j[k];
-                    if ((st[j] & kStMask) != 1) continue;
+                    if (!(st[j] & kStLive)) continue;
                     const uint64_t nw = Ch.new_work[k];
                     const uint64_t ttft_j = W[j] + nw;
                     if (!(Ch.ttft_i[k] > ttft_j && ttft_j < d.slo)) continue;
@@ -456,6 +463,7 @@ __global__ void __launch_bounds__(1024) k_rebalance(DevState d, uint32_t n, uint
             }
             __syncthreads();
             const uint32_t cnt0 = s_cnt;
+            uint64_t gone = 0;   // log records of the pending batch that leave i
             for (uint32_t t = threadIdx.x; t < s_nmv; t += blockDim.x) {
                 const uint32_t k = Ch.mv_k[t];
                 const uint32_t j = Ch.j[k];
@@ -479,12 +487,15 @@ __global__ void __launch_bounds__(1024) k_rebalance(DevState d, uint32_t n, uint
                     d.r_final[e.seq - seq0] = j;
                     d.info->final_dirty = 1;
                     const uint64_t nb = e.L / d.B;   // its log records move too
-                    atomicAdd(reinterpret_cast<unsigned long long *>(d.log_adv + i), (unsigned long long)-nb);
+                    gone += nb;
                     atomicAdd(reinterpret_cast<unsigned long long *>(d.log_adv + j), (unsigned long long)nb);
                     if (fresh) d.r_koff[e.seq - seq0] = e.koff;   // the commit writes its keys there
                 }
                 if (cnt0 + t < cap) out[cnt0 + t] = dm_migration{e.seq, i, j};
             }
+            gone = warp_sum_u64(gone);
+            if ((threadIdx.x & 31) == 0 && gone)
+                atomicAdd(reinterpret_cast<unsigned long long *>(d.log_adv + i), (unsigned long long)-gone);
             __syncthreads();
             if (fresh) {   // an earlier batch's moved request: its keys follow it
                 for (uint32_t t = 0; t < s_nmv; ++t) {

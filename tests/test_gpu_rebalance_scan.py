@@ -87,3 +87,33 @@ def test_hotspots_that_may_move_later(cost, seed):
     p.commit()
     p.check_state(tag="end")
     p.gpu.close()
+
+
+@pytest.mark.parametrize("share,slo", [((3000,), 1 << 30), ((3000, 900, 700), 20_000), ((1200, 1000, 900, 0, 40), 1 << 30),
+                                       ((2500, 2400), 1)])
+def test_hotspots_with_long_queues(share, slo):
+    """Hotspots with more than 256 entries for each hotspot (visited without a
+    scan) beside ones with fewer, over two batches."""
+    n = sum(share)
+    w = workload("tiny", n_instances=8, vnodes=32, slo_us=slo, batch=n, capacity=1 << 15, block_tokens=B,
+                 route_prefix_blocks=1)
+    p = Pair(w, max_instances=8, max_batch_tokens=1 << 20, max_touch=1 << 15, max_queue=1 << 14, choice_rule=5)
+    for i in range(8):
+        assert p.add(i) == 0
+    rng = np.random.default_rng(9)
+    starts = rng.integers(0, 32000, (400, B), dtype=np.uint32)
+    pos = np.array([p.ora.prompt_keys(x)[1] for x in starts], np.uint64)
+    c1 = p.ora.ring_owners(pos[:, 0].copy(), 0)
+    for t in (1, 2):
+        pick = np.concatenate([rng.choice(np.nonzero(c1 == i)[0], k) for i, k in enumerate(share) if k])
+        rng.shuffle(pick)
+        lens = rng.integers(B, 2 * B, n).astype(np.uint32)
+        off = np.arange(n, dtype=np.uint64) * np.uint64(2 * B)
+        tok = np.zeros((n, 2 * B), np.uint32)
+        tok[:, :B] = starts[pick]
+        p.route(tok.reshape(-1), off, lens, t)
+        moved = p.rebalance()
+        assert (moved > 0) == (slo > 1)
+        p.commit()
+    p.check_state(tag="end")
+    p.gpu.close()

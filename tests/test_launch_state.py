@@ -16,7 +16,7 @@ SRC = r"""
 #include <thread>
 #include <vector>
 
-static std::atomic<size_t> allowed[dm::kDevices];   // the made-up driver's setting per device
+static std::atomic<size_t> allowed[dm::kDevices];   // the made-up setting per device
 static std::atomic<int> calls;
 
 static int set_to(int dev, size_t bytes) {
